@@ -240,7 +240,7 @@ fe_status fe_ebe_apply_host(fe_mesh* mesh, int32_t R, fe_dtype dtype, const void
  *                  Deterministic: the same inputs give bitwise the same y.
  *                  fe_ebe_set_variant ignores tile_elems; fe_ebe_get_variant
  *                  returns the number of colours there;
- *   FE_EBE_WS      FP32 products only (R in {4, 8, 16, 32}; tile_elems * R / 2 a
+ *   FE_EBE_WS      FP32 products only (R in {4, 8, ..., 32}; tile_elems * R / 2 a
  *                  multiple of 32, at most 384): warp-specialised kernel, one
  *                  block per SM. Compute warps evaluate two cases of an element per
  *                  thread in paired FP32 instructions; staging warps bring in each

@@ -528,7 +528,7 @@ fe_status fe_ebe_set_variant(fe_mesh* m, int32_t R, fe_dtype dtype, int32_t vari
                    variant == FE_EBE_WS || variant == FE_EBE_DF_LEAN || variant == FE_EBE_WS2,
                "unknown variant %d", variant);
     FE_REQUIRE((variant != FE_EBE_WS && variant != FE_EBE_WS2) || (dtype == FE_F32 && ws_supported(R)),
-               "the warp-specialised kernel computes FP32 products for R in {4, 8, 16, 32}");
+               "the warp-specialised kernel computes FP32 products for R in {4, 8, ..., 32}");
     FE_REQUIRE((variant != FE_EBE_GATHER_DF && variant != FE_EBE_DF_LEAN) || (dtype == FE_F64 && df_supported(R)),
                "the float-float kernel computes FP64 products for R in {2, 4, 8, 16, 32}");
     FE_REQUIRE(variant != FE_EBE_GATHER_X2 || (dtype == FE_F32 && x2_supported(R)),

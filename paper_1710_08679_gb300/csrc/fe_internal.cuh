@@ -289,7 +289,7 @@ void build_colouring(fe_mesh* m, cudaStream_t s);
 // largest tile (elements) whose shared-memory footprint fits for (R, precision)
 bool tiled_fits(const fe_mesh* m, int tile_elems, int R, int is_f32, int kind);
 
-// Warp-specialised FP32 kernel (fe_ebe_ws.cu), R in {4, 8, 16, 32}
+// Warp-specialised FP32 kernel (fe_ebe_ws.cu), R in {4, 8, ..., 32}
 bool ws_supported(int R);
 const WsTiling* get_ws_tiling(fe_mesh* m, int tile_elems, int R, cudaStream_t s);
 // nth: threads per block, 512 (FE_EBE_WS, one block per SM) or 256 (FE_EBE_WS2, two)

@@ -1,0 +1,56 @@
+"""GPU parity, against the CPU oracle, of the kernels that are chosen by the size of a
+call: the FP64 direct product on both sides of its rule (four lanes per element, one
+lane per element and share of the cases), the sensitivities with an element's cases
+spread over lanes, the warp-specialised product for R that is no power of two, the
+4-case passes of the inner loops and the PCG iterations run as one device-side loop.
+
+Bars: those of the other parity tests (FP64 products 1e-12, FP32 products 2e-6 per
+case, sensitivities 1e-12, solutions 1e-6 from a solve to 1e-8).
+"""
+import numpy as np
+import pytest
+
+from _util import ensure_lib, rel_l2
+
+import oracle
+from paper_1710_08679_gb300 import meshgen as mg
+
+torch = pytest.importorskip("torch")
+
+TOL64, TOL32 = 1e-12, 2e-6
+DIRECT, WS, WS2 = 0, 6, 8
+
+MESHES = {
+    "box1": lambda: mg.plain_box(n=1, jitter=0.0),
+    "ragged": lambda: mg.crust_block(shape=(5, 3, 4), h=1000.0, jitter=0.15, seed=2)[0],
+    "box8": lambda: mg.plain_box(),
+    "crust20": lambda: mg.crust_block(shape=(20, 20, 10), h=1000.0, jitter=0.15, seed=5)[0],
+}
+
+
+@pytest.fixture(scope="module", params=list(MESHES))
+def case(request):
+    ensure_lib()
+    from paper_1710_08679_gb300 import fe
+    m = MESHES[request.param]()
+    return m, oracle.assemble(m), fe.Mesh.from_mesh(m)
+
+
+def cuda(a, dtype=torch.float64):
+    return torch.from_numpy(np.ascontiguousarray(a)).to(dtype).cuda()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("R,variant,tile", [(12, WS, 32), (12, WS2, 16), (20, WS, 16), (24, WS, 16), (24, WS2, 8),
+                                            (28, WS, 16)])
+def test_warp_specialised_product(case, R, variant, tile):
+    m, K, M = case
+    x = mg.random_vectors(m.n_nodes, R, seed=80 + R).astype(np.float32).astype(np.float64)
+    M.set_variant(R, "f32", variant, tile)
+    assert M.get_variant(R, "f32") == (variant, tile)
+    y = M.ebe(cuda(x, torch.float32))
+    M.device_status()   # no bounded wait of the kernel gave up
+    y = y.double().cpu().numpy()
+    ref = oracle.spmv(K, x)
+    for r in range(R):
+        assert rel_l2(y[:, r], ref[:, r]) <= TOL32, r
