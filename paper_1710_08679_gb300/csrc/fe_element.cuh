@@ -30,6 +30,17 @@ __host__ __device__ constexpr int edge_node(int a, int b) {
          : 9;  // (2,3)
 }
 
+// the same for loop indices (folds once the loops are unrolled); m itself for j = m
+__host__ __device__ __forceinline__ constexpr int edge_or_corner(int m, int j) {
+  return m == j ? m
+         : m + j == 1 ? 4
+         : m + j == 2 ? 6
+         : m + j == 4 ? 8
+         : m + j == 5 ? 9
+         : (m == 0 || j == 0) ? 7
+                              : 5;
+}
+
 template <typename T>
 struct ElemGeo {
   T g[4][3];  // gradients of the volume coordinates
@@ -162,19 +173,6 @@ __device__ __forceinline__ void elem_apply(const ElemGeo<T>& G, const T u[10][3]
   edge_out<0, 3>(s, G4, y);
   edge_out<1, 3>(s, G4, y);
   edge_out<2, 3>(s, G4, y);
-}
-
-// lambda^T K_e u for one case (adjoint element sensitivity), same arithmetic.
-template <typename T>
-__device__ __forceinline__ T elem_bilinear(const ElemGeo<T>& G, const T lam[10][3], const T u[10][3]) {
-  T y[10][3];
-  elem_apply(G, u, y);
-  T acc = T(0);
-#pragma unroll
-  for (int a = 0; a < 10; ++a)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) acc += lam[a][c] * y[a][c];
-  return acc;
 }
 
 }  // namespace fe

@@ -308,6 +308,27 @@ void grid_wait_selftest(const fe_mesh* m, long long cycles, cudaStream_t s);  //
 // Block Jacobi (fe_solver.cu)
 void build_block_jacobi(fe_mesh* m, cudaStream_t s);
 
+// Lanes an element's R cases are spread over in the FP64 kernels whose threads loop over
+// cases (a power of two at most 32). Each SM sub-partition runs its share of the warps
+// through its FP64 unit one instruction after the other, so the time is the largest
+// number of warps on one times a warp's FP64 instructions: `per_case` for each case and
+// about 150 for the geometry. More lanes even out the last round, fewer compute the
+// geometry less often.
+inline int f64_case_split(int64_t n_elem, int R, int per_case, int sms, int64_t* cost_out = nullptr) {
+  int best = 1;
+  int64_t best_cost = INT64_MAX;
+  for (int split = 1; split <= 32 && split < 2 * R; split *= 2) {
+    const int64_t warps = (n_elem * split + 31) / 32, units = 4 * (int64_t)sms;
+    const int64_t cost = ((warps + units - 1) / units) * ((int64_t)((R + split - 1) / split) * per_case + 150);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = split;
+    }
+  }
+  if (cost_out) *cost_out = best_cost;
+  return best;
+}
+
 // Adjoint (fe_adjoint.cu)
 void adjoint_grad(const fe_mesh* m, int R, const double* u, const double* lam, double* g, cudaStream_t s);
 

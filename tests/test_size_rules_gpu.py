@@ -41,6 +41,16 @@ def cuda(a, dtype=torch.float64):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("R", [1, 2, 5, 16, 33])
+def test_sensitivities(case, R):
+    m, _, M = case
+    u = mg.random_vectors(m.n_nodes, R, seed=60 + R)
+    lam = mg.random_vectors(m.n_nodes, R, seed=160 + R)
+    g = M.adjoint_grad(cuda(u), cuda(lam)).cpu().numpy()
+    assert rel_l2(g, oracle.adjoint_grad(m, u, lam)) <= TOL64
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("R,variant,tile", [(12, WS, 32), (12, WS2, 16), (20, WS, 16), (24, WS, 16), (24, WS2, 8),
                                             (28, WS, 16)])
 def test_warp_specialised_product(case, R, variant, tile):
