@@ -689,9 +689,7 @@ __global__ void s_pcg_alpha(Cases C) {
   C.D(D_ALPHA, r) = rho / g;
 }
 
-// PCG: beta = rho_new / rho, convergence and iteration cap
-__global__ void s_pcg_beta(Cases C, double tol, int max_it) {
-  const int r = threadIdx.x;
+__device__ __forceinline__ void pcg_beta_case(const Cases& C, int r, double tol, int max_it) {
   if (!C.I(I_ACTIVE, r)) {
     C.D(D_BETA, r) = 0.0;
     return;
@@ -865,6 +863,32 @@ __global__ void s_outer_check(Cases C, double tol, int max_outer) {
 struct InnerArgs {
   int64_t N;
   Cases C;
+// PCG: beta = rho_new / rho, convergence and iteration cap. With `use_loop` set, the
+// graph's while node repeats the iteration until a case leaves (a candidate for the
+// host to confirm, a breakdown, the cap): C.step() holds the cases active at the start.
+__global__ void s_pcg_beta(Cases C, double tol, int max_it, cudaGraphConditionalHandle loop, int use_loop) {
+  __shared__ int active;
+  const int r = threadIdx.x;
+  if (r == 0) active = 0;
+  __syncthreads();
+  pcg_beta_case(C, r, tol, max_it);
+  if (!use_loop) return;
+  if (C.I(I_ACTIVE, r)) atomicAdd(&active, 1);
+  __syncthreads();
+  if (r == 0) cudaGraphSetConditional(loop, active > 0 && active == C.step() ? 1u : 0u);
+}
+
+// PCG: counts the active cases before the while node
+__global__ void s_pcg_loop_begin(Cases C) {
+  __shared__ int active;
+  const int r = threadIdx.x;
+  if (r == 0) active = 0;
+  __syncthreads();
+  if (C.I(I_ACTIVE, r)) atomicAdd(&active, 1);
+  __syncthreads();
+  if (r == 0) C.step() = active;
+}
+
   const float* B;                                  // [N][9] inverse diagonal blocks
   const float* rb;
   float *ub, *eb, *pb, *qb;                        // [N][R][3]
@@ -1390,28 +1414,28 @@ static bool inner_loop_persistent(Solve& S, const Level& L) {
   return true;
 }
 
-static void inner_loop(Solve& S, const Level& L) {
-  if (inner_loop_persistent(S, L)) return;
-  level_apply(S, L, L.ub, L.qb, nullptr);
-  S.vec_on(L.N, *L.g, k_inner_resid, L.B, (const float*)L.rb, (const float*)L.qb, L.eb);
+// A while node in the graph being captured on S.s: its condition variable, set to
+// `start` at every launch of the graph, and the node, whose body is recorded on a
+// second stream into the node's own graph.
+static cudaGraphConditionalHandle while_handle(Solve& S, unsigned start) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  FE_CUDA(cudaStreamIsCapturing(S.s, &cs));
-  if (cs != cudaStreamCaptureStatusActive) {
-    // direct launches: all n steps are issued; those after the stop return at once
-    S.scal(s_inner_check, L.n, L.eps, L.f_rbn2, (cudaGraphConditionalHandle)0, 0);
-    for (int step = 0; step < L.n; ++step) inner_step(S, L, (cudaGraphConditionalHandle)0, 0);
-    return;
-  }
-  // recorded into a graph: a while node repeats one step while the stop test
-  // says go (the body is recorded on a second stream into the node's own graph)
   cudaGraph_t graph = nullptr;
   const cudaGraphNode_t* deps = nullptr;
   const cudaGraphEdgeData* edges = nullptr;
   size_t n_deps = 0;
-  cudaGraphConditionalHandle loop;
   FE_CUDA(cudaStreamGetCaptureInfo(S.s, &cs, nullptr, &graph, &deps, &edges, &n_deps));
-  FE_CUDA(cudaGraphConditionalHandleCreate(&loop, graph, 0, 0));
-  S.scal(s_inner_check, L.n, L.eps, L.f_rbn2, loop, 1);
+  cudaGraphConditionalHandle loop;
+  FE_CUDA(cudaGraphConditionalHandleCreate(&loop, graph, start, cudaGraphCondAssignDefault));
+  return loop;
+}
+
+template <typename Body>
+static void record_while(Solve& S, cudaGraphConditionalHandle loop, Body&& body_fn) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaGraph_t graph = nullptr;
+  const cudaGraphNode_t* deps = nullptr;
+  const cudaGraphEdgeData* edges = nullptr;
+  size_t n_deps = 0;
   FE_CUDA(cudaStreamGetCaptureInfo(S.s, &cs, nullptr, &graph, &deps, &edges, &n_deps));
   cudaGraphNodeParams np = {};
   np.type = cudaGraphNodeTypeConditional;
@@ -1425,7 +1449,7 @@ static void inner_loop(Solve& S, const Level& L) {
   FE_CUDA(cudaStreamBeginCaptureToGraph(S.w->body, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
   S.s = S.w->body;
   try {
-    inner_step(S, L, loop, 1);
+    body_fn();
   } catch (...) {
     S.s = outer;
     cudaGraph_t g;
@@ -1484,7 +1508,7 @@ static void fcg_iteration(Solve& S) {
 }
 
 // one PCG iteration
-static void pcg_iteration(Solve& S) {
+static void pcg_iteration(Solve& S, cudaGraphConditionalHandle loop = 0, int use_loop = 0) {
   SolverWork* w = S.w;
   const double* B64 = S.m->binv64.as<double>();
   ebe_apply<double>(S.m, S.R, w->p.as<double>(), w->q.as<double>(), S.s);
@@ -1493,7 +1517,7 @@ static void pcg_iteration(Solve& S) {
   S.scal(s_pcg_alpha);
   S.vec(k_pcg_update, B64, S.u, (const double*)w->p.as<double>(), w->r.as<double>(),
         (const double*)w->q.as<double>());
-  S.scal(s_pcg_beta, S.o.tol, S.o.max_outer);
+  S.scal(s_pcg_beta, S.o.tol, S.o.max_outer, loop, use_loop);
   S.vec(k_pcg_p, B64, (const double*)w->r.as<double>(), w->p.as<double>());
 }
 
@@ -1579,6 +1603,24 @@ static fe_status run_solve(fe_mesh* m, int R, const double* f, double* u, const 
       many->slot_case[(size_t)r] = many->next;
     }
   }
+static void inner_loop(Solve& S, const Level& L) {
+  if (inner_loop_persistent(S, L)) return;
+  level_apply(S, L, L.ub, L.qb, nullptr);
+  S.vec_on(L.N, *L.g, k_inner_resid, L.B, (const float*)L.rb, (const float*)L.qb, L.eb);
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  FE_CUDA(cudaStreamIsCapturing(S.s, &cs));
+  if (cs != cudaStreamCaptureStatusActive) {
+    // direct launches: all n steps are issued; those after the stop return at once
+    S.scal(s_inner_check, L.n, L.eps, L.f_rbn2, (cudaGraphConditionalHandle)0, 0);
+    for (int step = 0; step < L.n; ++step) inner_step(S, L, (cudaGraphConditionalHandle)0, 0);
+    return;
+  }
+  // recorded into a graph: a while node repeats one step while the stop test says go
+  const cudaGraphConditionalHandle loop = while_handle(S, 0);
+  S.scal(s_inner_check, L.n, L.eps, L.f_rbn2, loop, 1);
+  record_while(S, loop, [&] { inner_step(S, L, loop, 1); });
+}
+
   // start: u = P u, r = P f - K u, ||f||, ||r|| (the product is skipped when u = 0)
   S.scal(s_init);
   S.vec(k_prepare, m->nmask.as<uint8_t>(), f, u);
@@ -1591,13 +1633,15 @@ static fe_status run_solve(fe_mesh* m, int R, const double* f, double* u, const 
   FE_CUDA(cudaMemsetAsync(w->pb.ptr, 0, w->pb.bytes, s));
   if (pcg) S.vec(k_pcg_init, m->binv64.as<double>(), (const double*)w->r.as<double>(), w->p.as<double>());
 
-  // capture one iteration as a graph
+  // capture one iteration (PCG read at every iteration: the loop of them) as a graph
   cudaGraphExec_t exec = nullptr;
   if (o.use_graph) {
     cudaGraph_t graph;
     FE_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     try {
-      if (pcg) pcg_iteration(S); else fcg_iteration(S);
+      if (!pcg) fcg_iteration(S);
+      else if (o.check_every <= 1) pcg_loop(S);
+      else pcg_iteration(S);
     } catch (...) {
       cudaStreamEndCapture(s, &graph);
       throw;
@@ -1620,7 +1664,7 @@ static fe_status run_solve(fe_mesh* m, int R, const double* f, double* u, const 
       FE_CUDA(cudaStreamSynchronize(s));
       // confirm candidates with the true FP64 residual: one all-case product when
       // a quarter or more of the cases are candidates, else one product per case
-      bool any_active = false;
+      bool any_active = false, restart = false;
       int n_cand = 0;
       for (int c = 0; c < R; ++c) n_cand += hi[I_CAND * R + c] ? 1 : 0;
       const bool batched = R > 1 && 4 * n_cand >= R;
@@ -1639,6 +1683,16 @@ static fe_status run_solve(fe_mesh* m, int R, const double* f, double* u, const 
           const double rel = batched ? (fn2 > 0.0 ? std::sqrt(hd[D_RT2 * R + c] / fn2) : 0.0)
                                      : S.true_relres(c, fn2, true);
           int one = 1, zero = 0;
+// PCG iterations until a case leaves, recorded as one while node: the host reads the
+// flags when there is something to do and not after every iteration (a small mesh's
+// iteration takes less time than that read). Same iterates, and the same iteration
+// after which a case is confirmed, restarted or refilled.
+static void pcg_loop(Solve& S) {
+  S.scal(s_pcg_loop_begin);
+  const cudaGraphConditionalHandle loop = while_handle(S, 1);
+  record_while(S, loop, [&] { pcg_iteration(S, loop, 1); });
+}
+
           FE_CUDA(cudaMemcpyAsync(w->i.as<int>() + I_CAND * R + c, &zero, 4, cudaMemcpyHostToDevice, s));
           if (rel <= o.tol) {
             FE_CUDA(cudaMemcpyAsync(w->d.as<double>() + D_RELRES * R + c, &rel, 8, cudaMemcpyHostToDevice, s));
@@ -1646,7 +1700,7 @@ static fe_status run_solve(fe_mesh* m, int R, const double* f, double* u, const 
             // recursive residual drifted from the true one: continue from the true residual
             FE_CUDA(cudaMemcpyAsync(w->i.as<int>() + I_ACTIVE * R + c, &one, 4, cudaMemcpyHostToDevice, s));
             FE_CUDA(cudaMemcpyAsync(w->i.as<int>() + I_RESTART * R + c, &one, 4, cudaMemcpyHostToDevice, s));
-            any_active = true;
+            any_active = restart = true;
           }
           FE_CUDA(cudaStreamSynchronize(s));
         }
@@ -1691,11 +1745,11 @@ static fe_status run_solve(fe_mesh* m, int R, const double* f, double* u, const 
             s_slot_start<<<1, 1, 0, s>>>(S.C, r, pcg ? 1 : 0);
             FE_CHECK_LAUNCH();
             many->slot_case[(size_t)r] = nc;
-            any_active = true;
+            any_active = restart = true;
           }
         }
       }
-      if (pcg) {
+      if (pcg && restart) {
         // cases whose recursive residual drifted (or freshly loaded slots) restart CG from r
         FE_CUDA(cudaMemsetAsync(w->d.as<double>() + D_RHOA * R, 0, R * 8, s));
         S.vec(k_pcg_restart, m->binv64.as<double>(), (const double*)w->r.as<double>(), w->p.as<double>());

@@ -64,3 +64,25 @@ def test_warp_specialised_product(case, R, variant, tile):
     ref = oracle.spmv(K, x)
     for r in range(R):
         assert rel_l2(y[:, r], ref[:, r]) <= TOL32, r
+
+
+# cases that converge one after the other leave and re-enter the device-side loop
+@pytest.mark.gpu
+@pytest.mark.parametrize("R", [1, 3, 6])
+def test_pcg_loop_matches_single_iterations(R):
+    ensure_lib()
+    from paper_1710_08679_gb300 import fe
+    m = MESHES["ragged"]()
+    K = oracle.assemble(m)
+    f = mg.random_vectors(m.n_nodes, R, seed=9) * m.free[:, None, :]
+    ref = oracle.direct_solve(K, f)
+    M = fe.Mesh.from_mesh(m)
+    outer = []
+    for use_graph in (True, False):
+        u, stats, _ = M.solve(cuda(f), solver="pcg64", tol=1e-8, use_graph=use_graph)
+        assert rel_l2(u.cpu().numpy(), ref) <= 1e-6
+        assert all(s["relres"] <= 1e-8 for s in stats)
+        outer.append([s["outer"] for s in stats])
+    assert all(abs(a - b) <= 1 for a, b in zip(*outer)), outer   # sums in another order
+    _, stats, st = M.solve(cuda(f), solver="pcg64", tol=1e-8, max_outer=5, raise_on_fail=False)
+    assert st == fe.FE_ENOCONV and all(s["outer"] == 5 for s in stats)   # the cap ends the loop
