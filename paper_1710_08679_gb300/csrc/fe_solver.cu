@@ -716,6 +716,32 @@ __device__ __forceinline__ void pcg_beta_case(const Cases& C, int r, double tol,
   }
 }
 
+// PCG: beta = rho_new / rho, convergence and iteration cap. With `use_loop` set, the
+// graph's while node repeats the iteration until a case leaves (a candidate for the
+// host to confirm, a breakdown, the cap): C.step() holds the cases active at the start.
+__global__ void s_pcg_beta(Cases C, double tol, int max_it, cudaGraphConditionalHandle loop, int use_loop) {
+  __shared__ int active;
+  const int r = threadIdx.x;
+  if (r == 0) active = 0;
+  __syncthreads();
+  pcg_beta_case(C, r, tol, max_it);
+  if (!use_loop) return;
+  if (C.I(I_ACTIVE, r)) atomicAdd(&active, 1);
+  __syncthreads();
+  if (r == 0) cudaGraphSetConditional(loop, active > 0 && active == C.step() ? 1u : 0u);
+}
+
+// PCG: counts the active cases before the while node
+__global__ void s_pcg_loop_begin(Cases C) {
+  __shared__ int active;
+  const int r = threadIdx.x;
+  if (r == 0) active = 0;
+  __syncthreads();
+  if (C.I(I_ACTIVE, r)) atomicAdd(&active, 1);
+  __syncthreads();
+  if (r == 0) C.step() = active;
+}
+
 // FCG: start of one outer iteration
 __global__ void s_outer_begin(Cases C) {
   const int r = threadIdx.x;
@@ -863,32 +889,6 @@ __global__ void s_outer_check(Cases C, double tol, int max_outer) {
 struct InnerArgs {
   int64_t N;
   Cases C;
-// PCG: beta = rho_new / rho, convergence and iteration cap. With `use_loop` set, the
-// graph's while node repeats the iteration until a case leaves (a candidate for the
-// host to confirm, a breakdown, the cap): C.step() holds the cases active at the start.
-__global__ void s_pcg_beta(Cases C, double tol, int max_it, cudaGraphConditionalHandle loop, int use_loop) {
-  __shared__ int active;
-  const int r = threadIdx.x;
-  if (r == 0) active = 0;
-  __syncthreads();
-  pcg_beta_case(C, r, tol, max_it);
-  if (!use_loop) return;
-  if (C.I(I_ACTIVE, r)) atomicAdd(&active, 1);
-  __syncthreads();
-  if (r == 0) cudaGraphSetConditional(loop, active > 0 && active == C.step() ? 1u : 0u);
-}
-
-// PCG: counts the active cases before the while node
-__global__ void s_pcg_loop_begin(Cases C) {
-  __shared__ int active;
-  const int r = threadIdx.x;
-  if (r == 0) active = 0;
-  __syncthreads();
-  if (C.I(I_ACTIVE, r)) atomicAdd(&active, 1);
-  __syncthreads();
-  if (r == 0) C.step() = active;
-}
-
   const float* B;                                  // [N][9] inverse diagonal blocks
   const float* rb;
   float *ub, *eb, *pb, *qb;                        // [N][R][3]
@@ -1461,6 +1461,24 @@ static void record_while(Solve& S, cudaGraphConditionalHandle loop, Body&& body_
   FE_CUDA(cudaStreamUpdateCaptureDependencies(S.s, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
 }
 
+static void inner_loop(Solve& S, const Level& L) {
+  if (inner_loop_persistent(S, L)) return;
+  level_apply(S, L, L.ub, L.qb, nullptr);
+  S.vec_on(L.N, *L.g, k_inner_resid, L.B, (const float*)L.rb, (const float*)L.qb, L.eb);
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  FE_CUDA(cudaStreamIsCapturing(S.s, &cs));
+  if (cs != cudaStreamCaptureStatusActive) {
+    // direct launches: all n steps are issued; those after the stop return at once
+    S.scal(s_inner_check, L.n, L.eps, L.f_rbn2, (cudaGraphConditionalHandle)0, 0);
+    for (int step = 0; step < L.n; ++step) inner_step(S, L, (cudaGraphConditionalHandle)0, 0);
+    return;
+  }
+  // recorded into a graph: a while node repeats one step while the stop test says go
+  const cudaGraphConditionalHandle loop = while_handle(S, 0);
+  S.scal(s_inner_check, L.n, L.eps, L.f_rbn2, loop, 1);
+  record_while(S, loop, [&] { inner_step(S, L, loop, 1); });
+}
+
 // the FCG outer iteration (Algorithm 1(a)): inner loop level 1 when the coarse
 // level is on, with inner loop level 2 before it when the aggregation level is on
 static void fcg_iteration(Solve& S) {
@@ -1519,6 +1537,16 @@ static void pcg_iteration(Solve& S, cudaGraphConditionalHandle loop = 0, int use
         (const double*)w->q.as<double>());
   S.scal(s_pcg_beta, S.o.tol, S.o.max_outer, loop, use_loop);
   S.vec(k_pcg_p, B64, (const double*)w->r.as<double>(), w->p.as<double>());
+}
+
+// PCG iterations until a case leaves, recorded as one while node: the host reads the
+// flags when there is something to do and not after every iteration (a small mesh's
+// iteration takes less time than that read). Same iterates, and the same iteration
+// after which a case is confirmed, restarted or refilled.
+static void pcg_loop(Solve& S) {
+  S.scal(s_pcg_loop_begin);
+  const cudaGraphConditionalHandle loop = while_handle(S, 1);
+  record_while(S, loop, [&] { pcg_iteration(S, loop, 1); });
 }
 
 // Many-case mode: n_cases right-hand sides stream through R slots. f and u of
@@ -1603,24 +1631,6 @@ static fe_status run_solve(fe_mesh* m, int R, const double* f, double* u, const 
       many->slot_case[(size_t)r] = many->next;
     }
   }
-static void inner_loop(Solve& S, const Level& L) {
-  if (inner_loop_persistent(S, L)) return;
-  level_apply(S, L, L.ub, L.qb, nullptr);
-  S.vec_on(L.N, *L.g, k_inner_resid, L.B, (const float*)L.rb, (const float*)L.qb, L.eb);
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  FE_CUDA(cudaStreamIsCapturing(S.s, &cs));
-  if (cs != cudaStreamCaptureStatusActive) {
-    // direct launches: all n steps are issued; those after the stop return at once
-    S.scal(s_inner_check, L.n, L.eps, L.f_rbn2, (cudaGraphConditionalHandle)0, 0);
-    for (int step = 0; step < L.n; ++step) inner_step(S, L, (cudaGraphConditionalHandle)0, 0);
-    return;
-  }
-  // recorded into a graph: a while node repeats one step while the stop test says go
-  const cudaGraphConditionalHandle loop = while_handle(S, 0);
-  S.scal(s_inner_check, L.n, L.eps, L.f_rbn2, loop, 1);
-  record_while(S, loop, [&] { inner_step(S, L, loop, 1); });
-}
-
   // start: u = P u, r = P f - K u, ||f||, ||r|| (the product is skipped when u = 0)
   S.scal(s_init);
   S.vec(k_prepare, m->nmask.as<uint8_t>(), f, u);
@@ -1683,16 +1693,6 @@ static void inner_loop(Solve& S, const Level& L) {
           const double rel = batched ? (fn2 > 0.0 ? std::sqrt(hd[D_RT2 * R + c] / fn2) : 0.0)
                                      : S.true_relres(c, fn2, true);
           int one = 1, zero = 0;
-// PCG iterations until a case leaves, recorded as one while node: the host reads the
-// flags when there is something to do and not after every iteration (a small mesh's
-// iteration takes less time than that read). Same iterates, and the same iteration
-// after which a case is confirmed, restarted or refilled.
-static void pcg_loop(Solve& S) {
-  S.scal(s_pcg_loop_begin);
-  const cudaGraphConditionalHandle loop = while_handle(S, 1);
-  record_while(S, loop, [&] { pcg_iteration(S, loop, 1); });
-}
-
           FE_CUDA(cudaMemcpyAsync(w->i.as<int>() + I_CAND * R + c, &zero, 4, cudaMemcpyHostToDevice, s));
           if (rel <= o.tol) {
             FE_CUDA(cudaMemcpyAsync(w->d.as<double>() + D_RELRES * R + c, &rel, 8, cudaMemcpyHostToDevice, s));
