@@ -80,7 +80,8 @@ __device__ __forceinline__ void load_geometry(const MeshView<T>& M, int64_t e, c
 // ---------------------------------------------------------------------------
 // direct kernel: thread = (element, case)
 // ---------------------------------------------------------------------------
-// FP32: at most 128 registers so that two 256-thread blocks fit per SM
+// FP32 (FP64: ebe_direct_f64_kernel): at most 128 registers so that two 256-thread blocks
+// fit per SM
 template <typename T>
 struct MinBlocks {
   static constexpr int value = sizeof(T) == 4 ? 2 : 1;
@@ -90,8 +91,8 @@ template <typename T>
 __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) ebe_direct_kernel(MeshView<T> M, int R, const uint16_t* __restrict__ own,
                                                               const T* __restrict__ x, T* __restrict__ y,
                                                               const int* __restrict__ skip) {
-  if (skip && *skip) return;
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (skip && *skip) return;
   if (gid >= M.n_elem * R) return;
   const int64_t e = gid / R;
   const int r = (int)(gid - e * R);
@@ -120,6 +121,194 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) ebe_direct_kern
         atomicAdd(ya + c, yl[a][c]);
       else if ((ow >> a) & 1)   // constrained DOF: (I - P) x, written once by the node's owner element
         ya[c] = __ldg(x + ((int64_t)nd[a] * R + r) * 3 + c);
+    }
+  }
+}
+
+// FP64 direct kernel: thread = (element, share of the cases); lane `part` of an
+// element's `split` lanes takes cases part, part + split, ... Bound by the FP64 pipe (1/61
+// of FP32), so the geometry, a fifth of a case's FP64 instructions, is computed once
+// per thread, and blocks of one warp fill the SMs evenly.
+__global__ void __launch_bounds__(32) ebe_direct_f64_kernel(MeshView<double> M, int R, int split,
+                                                            const uint16_t* __restrict__ own,
+                                                            const double* __restrict__ x, double* __restrict__ y,
+                                                            const int* __restrict__ skip) {
+  const int64_t gid = blockIdx.x * (int64_t)32 + threadIdx.x;
+  const int64_t e = gid / split;
+  const int part = (int)(gid - e * split);
+  if ((skip && *skip) || e >= M.n_elem) return;
+  int nd[10];
+  load_conn<double>(M.conn, e, nd);
+  ElemGeo<double> G;
+  load_geometry(M, e, nd, G);
+  const ElemCases<double> C(G);
+  unsigned mk = 0;
+#pragma unroll
+  for (int a = 0; a < 10; ++a) mk |= ((unsigned)__ldg(M.nmask + nd[a]) & 7u) << (3 * a);
+  const int ow = __ldg(own + e);
+  for (int r = part; r < R; r += split) {
+    double u[10][3], yl[10][3];
+#pragma unroll
+    for (int a = 0; a < 10; ++a) {
+      const double* xa = x + ((int64_t)nd[a] * R + r) * 3;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) u[a][c] = ((mk >> (3 * a + c)) & 1) ? __ldg(xa + c) : 0.0;
+    }
+    elem_apply_case(C, u, yl);
+#pragma unroll
+    for (int a = 0; a < 10; ++a) {
+      const int64_t o = ((int64_t)nd[a] * R + r) * 3;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        if ((mk >> (3 * a + c)) & 1)
+          atomicAdd(y + o + c, yl[a][c]);
+        else if ((ow >> a) & 1)   // constrained DOF: (I - P) x, written once by the node's owner element
+          y[o + c] = __ldg(x + o + c);
+      }
+    }
+  }
+}
+
+// FP64 direct kernel for few items: four lanes per (element, case), lane m = corner m. A
+// warp's FP64 instruction occupies its SM sub-partition for some 60 cycles whatever the
+// other sub-partitions do, so with fewer warps than sub-partitions (608) the time is one
+// warp's FP64 instruction count: 588 with a lane per element. Here a lane forms its
+// corner's gradient (one of the three quotients 1/det, lam, mu per lane), stress s_m,
+// corner output and its terms T_m g_l of the three edges at its corner: about 200. One case
+// on the 3,072 elements of the 8^3 box: 25 us with a lane per element (kernel); the whole
+// product 28.3 (gather kernel, the fastest before) -> 18.1 us; a 172-step PCG solve 7.6 -> 5.1 ms.
+__global__ void __launch_bounds__(64) ebe_corner_f64_kernel(MeshView<double> M, int R,
+                                                            const uint16_t* __restrict__ own,
+                                                            const double* __restrict__ x, double* __restrict__ y,
+                                                            const int* __restrict__ skip) {
+  if (skip && *skip) return;
+  constexpr unsigned kAll = 0xffffffffu;
+  const int64_t gid = blockIdx.x * (int64_t)64 + threadIdx.x;
+  const int m = threadIdx.x & 3;
+  const int64_t item = gid >> 2;
+  const bool work = item < M.n_elem * R;
+  const int64_t it = work ? item : 0;   // idle lanes compute item 0 and write nothing
+  const int64_t e = it / R;
+  const int r = (int)(it - e * R);
+  // lane m's corners in the order m, m + 1, m + 2, m + 3 (mod 4): an odd permutation of
+  // (0, 1, 2, 3) for odd m, which the sign of the determinant follows
+  int nc[4], ne[3];   // corner nodes, edge nodes (m, m + 1), (m, m + 2), (m, m + 3)
+  double xc[4][3];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    nc[k] = __ldg(M.conn + 10 * e + ((m + k) & 3));
+    if (k > 0) ne[k - 1] = __ldg(M.conn + 10 * e + edge_or_corner(m, (m + k) & 3));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) xc[k][i] = __ldg(M.xyz + 3 * (int64_t)nc[k] + i);
+  }
+  double u[4][3], w[3][3];   // corners, edges
+  int mc[4], me[3];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    mc[k] = __ldg(M.nmask + nc[k]);
+    const double* xa = x + ((int64_t)nc[k] * R + r) * 3;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) u[k][c] = ((mc[k] >> c) & 1) ? __ldg(xa + c) : 0.0;
+    if (k > 0) {
+      me[k - 1] = __ldg(M.nmask + ne[k - 1]);
+      const double* xe = x + ((int64_t)ne[k - 1] * R + r) * 3;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) w[k - 1][c] = ((me[k - 1] >> c) & 1) ? __ldg(xe + c) : 0.0;
+    }
+  }
+  // g_m: normal of the opposite face over the determinant
+  double d2[3], d3[3], dm[3], n[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    d2[i] = xc[2][i] - xc[1][i];
+    d3[i] = xc[3][i] - xc[1][i];
+    dm[i] = xc[0][i] - xc[1][i];
+  }
+  n[0] = d2[1] * d3[2] - d2[2] * d3[1];
+  n[1] = d2[2] * d3[0] - d2[0] * d3[2];
+  n[2] = d2[0] * d3[1] - d2[1] * d3[0];
+  const double dets = dm[0] * n[0] + dm[1] * n[1] + dm[2] * n[2];
+  const double det = fabs(dets);
+  const double E = __ldg(M.mat + 2 * e), nu = __ldg(M.mat + 2 * e + 1), onu = 1.0 + nu;
+  // lanes 0, 1: mu, lam; lanes 2, 3: the reciprocal determinant
+  const double num = m == 0 ? E : m == 1 ? E * nu : 1.0;
+  const double den = m == 0 ? 2.0 * onu : m == 1 ? onu * (1.0 - 2.0 * nu) : det;
+  const double quo = num / den;
+  const double c4 = __shfl_sync(kAll, det, 0, 4) * (1.0 / 30.0);   // V/5
+  const double mu = __shfl_sync(kAll, quo, 0, 4) * c4, lam = __shfl_sync(kAll, quo, 1, 4) * c4;
+  double inv = __shfl_sync(kAll, quo, 2, 4);
+  if (dets < 0.0) inv = -inv;
+  double g[4][3];   // g of corners m, m + 1, m + 2, m + 3
+#pragma unroll
+  for (int i = 0; i < 3; ++i) g[0][i] = n[i] * inv;
+#pragma unroll
+  for (int k = 1; k < 4; ++k)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) g[k][i] = __shfl_sync(kAll, g[0][i], (m + k) & 3, 4);
+  // s_m
+  double H[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const double v = 3.0 * u[0][a];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) H[a][b] = v * g[0][b];
+  }
+#pragma unroll
+  for (int k = 1; k < 4; ++k)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const double v = 4.0 * w[k - 1][a] - u[k][a];
+#pragma unroll
+      for (int b = 0; b < 3; ++b) H[a][b] += v * g[k][b];
+    }
+  const double lt = lam * (H[0][0] + H[1][1] + H[2][2]), two_mu = 2.0 * mu;
+  double s[6] = {lt + two_mu * H[0][0], lt + two_mu * H[1][1], lt + two_mu * H[2][2],
+                 mu * (H[1][2] + H[2][1]), mu * (H[0][2] + H[2][0]), mu * (H[0][1] + H[1][0])};
+  double A[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    double S = s[q] + __shfl_xor_sync(kAll, s[q], 1);
+    S += __shfl_xor_sync(kAll, S, 2);
+    A[q] = s[q] - 0.25 * S;
+    s[q] += S;   // T_m
+  }
+  const int ow = __ldg(own + e);
+  double o[3];
+  sym_mv(A, g[0], o);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int64_t at = ((int64_t)nc[0] * R + r) * 3 + c;
+    if (work) {
+      if ((mc[0] >> c) & 1)
+        atomicAdd(y + at, o[c]);
+      else if ((ow >> m) & 1)   // constrained DOF: (I - P) x, written once by the node's owner element
+        y[at] = __ldg(x + at);
+    }
+  }
+  // edges: this lane's terms T_m g_l for l = m + 1, m + 2, m + 3, and the other end's from
+  // its lane (whose third, second and first they are). Lane m writes edge (m, m + 1), lanes
+  // 0 and 1 edges (0, 2) and (1, 3).
+  double t1[3], t2[3], t3[3];
+  sym_mv(s, g[1], t1);
+  sym_mv(s, g[2], t2);
+  sym_mv(s, g[3], t3);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    t1[c] += __shfl_sync(kAll, t3[c], (m + 1) & 3, 4);
+    t2[c] += __shfl_xor_sync(kAll, t2[c], 2);
+  }
+#pragma unroll
+  for (int k = 1; k < 3; ++k) {
+    const int a = edge_or_corner(m, (m + k) & 3);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int64_t at = ((int64_t)ne[k - 1] * R + r) * 3 + c;
+      if (work && (k == 1 || m < 2)) {
+        if ((me[k - 1] >> c) & 1)
+          atomicAdd(y + at, k == 1 ? t1[c] : t2[c]);
+        else if ((ow >> a) & 1)
+          y[at] = __ldg(x + at);
+      }
     }
   }
 }
@@ -1186,10 +1375,29 @@ size_t tiled_smem_bytes(int max_nodes, int tile_elems, int R) {
 template <typename T>
 static void launch_direct(const fe_mesh* m, int R, const T* x, T* y, cudaStream_t s, const int* skip) {
   const MeshView<T> M = m->view<T>();
-  const int64_t total = M.n_elem * R;
-  const int64_t blocks = (total + kThreads - 1) / kThreads;
-  ebe_direct_kernel<T><<<(unsigned)blocks, kThreads, 0, s>>>(M, R, m->own_elem.as<uint16_t>(), x, y, skip);
-  FE_CHECK_LAUNCH();
+  int sms = 0;
+  FE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
+  if constexpr (sizeof(T) == 8) {
+    int64_t cost = 0;
+    const int split = f64_case_split(M.n_elem, R, 438, sms, &cost);
+    const int64_t lanes = 4 * M.n_elem * R, units = 4 * (int64_t)sms;
+    if (((lanes + 31) / 32 + units - 1) / units * 200 < cost) {
+      ebe_corner_f64_kernel<<<(unsigned)((lanes + 63) / 64), 64, 0, s>>>(M, R, m->own_elem.as<uint16_t>(), x, y, skip);
+    FE_CHECK_LAUNCH();
+      return;
+    }
+    const int64_t blocks = (M.n_elem * split + 31) / 32;
+    ebe_direct_f64_kernel<<<(unsigned)(blocks), 32, 0, s>>>(M, R, split, m->own_elem.as<uint16_t>(), x, y, skip);
+    FE_CHECK_LAUNCH();
+  } else {
+    // smaller blocks where the largest would leave SMs with less than four of them
+    const int64_t total = M.n_elem * R;
+    int tpb = kThreads;
+    while (tpb > 32 && total < (int64_t)tpb * sms * 4) tpb /= 2;
+    const int64_t blocks = (total + tpb - 1) / tpb;
+    ebe_direct_kernel<T><<<(unsigned)(blocks), tpb, 0, s>>>(M, R, m->own_elem.as<uint16_t>(), x, y, skip);
+    FE_CHECK_LAUNCH();
+  }
 }
 
 template <typename T>

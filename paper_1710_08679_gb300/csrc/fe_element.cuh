@@ -175,4 +175,81 @@ __device__ __forceinline__ void elem_apply(const ElemGeo<T>& G, const T u[10][3]
   edge_out<2, 3>(s, G4, y);
 }
 
+// Element data for several cases of one element: what elem_apply computes per case from
+// the geometry alone (3 g, and V/5 folded into the Lame constants) formed once.
+template <typename T>
+struct ElemCases {
+  T g[4][3], g3[4][3];
+  T lam, mu, two_mu;   // times V/5
+  __device__ __forceinline__ explicit ElemCases(const ElemGeo<T>& G) {
+    const T c4 = T(4) * G.c;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        g[k][i] = G.g[k][i];
+        g3[k][i] = T(3) * G.g[k][i];
+      }
+    lam = G.lam * c4;
+    mu = G.mu * c4;
+    two_mu = T(2) * mu;
+  }
+};
+
+// y = K_e u for one case from the element's case-independent data: 438 operations, most
+// of them multiply-adds (elem_apply: 463).
+template <typename T>
+__device__ __forceinline__ void elem_apply_case(const ElemCases<T>& G, const T u[10][3], T y[10][3]) {
+  T s[4][6];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    T H[3][3];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      T v[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) v[a] = j == m ? u[m][a] : T(4) * u[edge_or_corner(m, j)][a] - u[j][a];
+      const T* w = j == m ? G.g3[j] : G.g[j];
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) H[a][b] = j == 0 ? v[a] * w[b] : H[a][b] + v[a] * w[b];
+    }
+    const T lt = G.lam * (H[0][0] + H[1][1] + H[2][2]);
+    s[m][0] = lt + G.two_mu * H[0][0];
+    s[m][1] = lt + G.two_mu * H[1][1];
+    s[m][2] = lt + G.two_mu * H[2][2];
+    s[m][3] = G.mu * (H[1][2] + H[2][1]);
+    s[m][4] = G.mu * (H[0][2] + H[2][0]);
+    s[m][5] = G.mu * (H[0][1] + H[1][0]);
+  }
+  T S[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) S[q] = (s[0][q] + s[1][q]) + (s[2][q] + s[3][q]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    T A[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) A[q] = s[k][q] - T(0.25) * S[q];
+    sym_mv(A, G.g[k], y[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int q = 0; q < 6; ++q) s[k][q] += S[q];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int l = k + 1; l < 4; ++l) {
+      const T* a = s[k];
+      const T* b = s[l];
+      const T* g = G.g[l];
+      const T* h = G.g[k];
+      T* w = y[edge_or_corner(k, l)];
+      w[0] = a[0] * g[0] + a[5] * g[1] + a[4] * g[2] + b[0] * h[0] + b[5] * h[1] + b[4] * h[2];
+      w[1] = a[5] * g[0] + a[1] * g[1] + a[3] * g[2] + b[5] * h[0] + b[1] * h[1] + b[3] * h[2];
+      w[2] = a[4] * g[0] + a[3] * g[1] + a[2] * g[2] + b[4] * h[0] + b[3] * h[1] + b[2] * h[2];
+    }
+}
+
 }  // namespace fe

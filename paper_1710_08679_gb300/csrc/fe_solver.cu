@@ -92,7 +92,7 @@ void free_solver_work(fe_mesh* m) {
 // ---------------------------------------------------------------------------
 // launch geometry for [N][R][3] vector kernels: blocks of K*R threads, thread
 // (j, r) = (threadIdx.x / R, threadIdx.x % R) handles node n = block*K + j
-// (grid-stride) and case r. K is the largest power of two with K*R <= 256.
+// (grid-stride) and case r. K is a power of two, the largest with K*R <= 256 on large meshes.
 // ---------------------------------------------------------------------------
 struct VGeom {
   int R, K, tpb;
@@ -104,6 +104,9 @@ static VGeom vgeom(int64_t N, int R, int sms) {
   g.R = R;
   g.K = 1;
   while (g.K * 2 * R <= 256) g.K *= 2;
+  // small meshes: blocks down to one warp until every SM has one (FP64 instructions of one
+  // SM's warps queue behind each other)
+  while (g.K > 1 && g.K * R > 32 && (N + g.K - 1) / g.K < sms) g.K /= 2;
   g.tpb = g.K * R;
   const int64_t need = (N + g.K - 1) / g.K;
   const int64_t cap = (int64_t)sms * 8;

@@ -40,6 +40,22 @@ def cuda(a, dtype=torch.float64):
     return torch.from_numpy(np.ascontiguousarray(a)).to(dtype).cuda()
 
 
+# from 6 items (box1, R = 1) over one warp per SM sub-partition (box8) to many (crust20)
+@pytest.mark.gpu
+@pytest.mark.parametrize("R", [1, 2, 5, 7, 17])
+def test_direct_fp64_product(case, R):
+    m, K, M = case
+    x = mg.random_vectors(m.n_nodes, R, seed=40 + R)
+    M.set_variant(R, "f64", DIRECT, 48)
+    y = M.ebe(cuda(x)).cpu().numpy()
+    ref = oracle.spmv(K, x)
+    for r in range(R):
+        assert rel_l2(y[:, r], ref[:, r]) <= TOL64, r
+    fixed = m.free == 0
+    for r in range(R):   # constrained DOFs: (I - P) x
+        assert np.array_equal(y[:, r][fixed], x[:, r][fixed])
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("R", [1, 2, 5, 16, 33])
 def test_sensitivities(case, R):
