@@ -42,9 +42,15 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// The zero pass lets the product kernel behind it start while it runs (launch_behind_zero);
+// that kernel loads and computes, and waits here before it first writes y. (No effect on
+// kernels launched in the ordinary way.)
+__device__ __forceinline__ void wait_for_zero() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // y = 0 with 16-byte stores (write-only pass before the atomic accumulation)
 template <typename T>
 __global__ void __launch_bounds__(kThreads) zero_kernel(int64_t n, T* __restrict__ y, const int* __restrict__ skip) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (skip && *skip) return;
   const int64_t n4 = n * (int64_t)sizeof(T) / 16;
   float4* y4 = reinterpret_cast<float4*>(y);
@@ -92,8 +98,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) ebe_direct_kern
                                                               const T* __restrict__ x, T* __restrict__ y,
                                                               const int* __restrict__ skip) {
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (skip && *skip) return;
-  if (gid >= M.n_elem * R) return;
+  if ((skip && *skip) || gid >= M.n_elem * R) return wait_for_zero();
   const int64_t e = gid / R;
   const int r = (int)(gid - e * R);
   int nd[10];
@@ -112,6 +117,7 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) ebe_direct_kern
   T yl[10][3];
   elem_apply(G, u, yl);
   const int ow = __ldg(own + e);
+  wait_for_zero();
 #pragma unroll
   for (int a = 0; a < 10; ++a) {
     T* ya = y + ((int64_t)nd[a] * R + r) * 3;
@@ -136,7 +142,7 @@ __global__ void __launch_bounds__(32) ebe_direct_f64_kernel(MeshView<double> M, 
   const int64_t gid = blockIdx.x * (int64_t)32 + threadIdx.x;
   const int64_t e = gid / split;
   const int part = (int)(gid - e * split);
-  if ((skip && *skip) || e >= M.n_elem) return;
+  if ((skip && *skip) || e >= M.n_elem) return wait_for_zero();
   int nd[10];
   load_conn<double>(M.conn, e, nd);
   ElemGeo<double> G;
@@ -155,6 +161,7 @@ __global__ void __launch_bounds__(32) ebe_direct_f64_kernel(MeshView<double> M, 
       for (int c = 0; c < 3; ++c) u[a][c] = ((mk >> (3 * a + c)) & 1) ? __ldg(xa + c) : 0.0;
     }
     elem_apply_case(C, u, yl);
+    wait_for_zero();
 #pragma unroll
     for (int a = 0; a < 10; ++a) {
       const int64_t o = ((int64_t)nd[a] * R + r) * 3;
@@ -181,7 +188,7 @@ __global__ void __launch_bounds__(64) ebe_corner_f64_kernel(MeshView<double> M, 
                                                             const uint16_t* __restrict__ own,
                                                             const double* __restrict__ x, double* __restrict__ y,
                                                             const int* __restrict__ skip) {
-  if (skip && *skip) return;
+  if (skip && *skip) return wait_for_zero();
   constexpr unsigned kAll = 0xffffffffu;
   const int64_t gid = blockIdx.x * (int64_t)64 + threadIdx.x;
   const int m = threadIdx.x & 3;
@@ -275,6 +282,7 @@ __global__ void __launch_bounds__(64) ebe_corner_f64_kernel(MeshView<double> M, 
   const int ow = __ldg(own + e);
   double o[3];
   sym_mv(A, g[0], o);
+  wait_for_zero();
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const int64_t at = ((int64_t)nc[0] * R + r) * 3 + c;
@@ -552,7 +560,7 @@ __global__ void __launch_bounds__(kThreads) ebe_gather_kernel(MeshView<T> M, int
   using VT = typename Vec16<T>::type;
   constexpr int VR = C::VR, V = C::V, S = C::S;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (skip && *skip) return;
+  if (skip && *skip) return wait_for_zero();
   const int64_t tile = blockIdx.x;
   const int nb = __ldg(node_ptr + tile);
   const int nn = __ldg(node_ptr + tile + 1) - nb;
@@ -661,6 +669,7 @@ __global__ void __launch_bounds__(kThreads) ebe_gather_kernel(MeshView<T> M, int
   }
   __syncthreads();
 
+  wait_for_zero();
   // ---- phase 3
   if constexpr (C::VEC) {
     constexpr int CPN = VR / V;
@@ -1219,7 +1228,8 @@ __global__ void __launch_bounds__(kThreads) ebe_pipe_df_kernel(int64_t n_tiles, 
 // split, slots and node sums of ebe_pipe_df_kernel, with
 //  * elem_apply_df_lean: node values and geometry read from shared memory where
 //    they are used and outputs stored as they are formed, so the product fits in
-//    128 registers per thread;
+//    128 registers per thread; paired FP32 instructions over corners of the element
+//    (and over two values of a node in the sums);
 //  * one input stage: the next tile's rows are copied while this tile's node
 //    sums run (they read only the slots), which halves that buffer.
 // Two 256-thread blocks per SM then overlap each other's phases (split, element
@@ -1372,6 +1382,26 @@ size_t tiled_smem_bytes(int max_nodes, int tile_elems, int R) {
 
 }  // namespace
 
+// Launches a product kernel behind the zero pass on the same stream: it may start while the
+// zero pass runs (programmatic dependent launch), which hides a launch and its latency on
+// small meshes. Not while a graph is captured: ordinary dependencies there.
+template <typename... P, typename... A>
+static void launch_behind_zero(void (*kernel)(P...), int64_t grid, int threads, size_t smem, cudaStream_t s, A... args) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  FE_CUDA(cudaStreamIsCapturing(s, &cs));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cs == cudaStreamCaptureStatusNone ? 1 : 0;
+  FE_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+}
+
 template <typename T>
 static void launch_direct(const fe_mesh* m, int R, const T* x, T* y, cudaStream_t s, const int* skip) {
   const MeshView<T> M = m->view<T>();
@@ -1382,21 +1412,18 @@ static void launch_direct(const fe_mesh* m, int R, const T* x, T* y, cudaStream_
     const int split = f64_case_split(M.n_elem, R, 438, sms, &cost);
     const int64_t lanes = 4 * M.n_elem * R, units = 4 * (int64_t)sms;
     if (((lanes + 31) / 32 + units - 1) / units * 200 < cost) {
-      ebe_corner_f64_kernel<<<(unsigned)((lanes + 63) / 64), 64, 0, s>>>(M, R, m->own_elem.as<uint16_t>(), x, y, skip);
-    FE_CHECK_LAUNCH();
+      launch_behind_zero(ebe_corner_f64_kernel, (lanes + 63) / 64, 64, 0, s, M, R, m->own_elem.as<uint16_t>(), x, y, skip);
       return;
     }
     const int64_t blocks = (M.n_elem * split + 31) / 32;
-    ebe_direct_f64_kernel<<<(unsigned)(blocks), 32, 0, s>>>(M, R, split, m->own_elem.as<uint16_t>(), x, y, skip);
-    FE_CHECK_LAUNCH();
+    launch_behind_zero(ebe_direct_f64_kernel, blocks, 32, 0, s, M, R, split, m->own_elem.as<uint16_t>(), x, y, skip);
   } else {
     // smaller blocks where the largest would leave SMs with less than four of them
     const int64_t total = M.n_elem * R;
     int tpb = kThreads;
     while (tpb > 32 && total < (int64_t)tpb * sms * 4) tpb /= 2;
     const int64_t blocks = (total + tpb - 1) / tpb;
-    ebe_direct_kernel<T><<<(unsigned)(blocks), tpb, 0, s>>>(M, R, m->own_elem.as<uint16_t>(), x, y, skip);
-    FE_CHECK_LAUNCH();
+    launch_behind_zero(ebe_direct_kernel<T>, blocks, tpb, 0, s, M, R, m->own_elem.as<uint16_t>(), x, y, skip);
   }
 }
 
@@ -1455,10 +1482,9 @@ static void launch_gather_r(const fe_mesh* m, const Tiling& t, const T* x, T* y,
   FE_REQUIRE(smem <= (size_t)max_smem_optin(m->device), "gather tile of %d elements needs %zu B shared memory",
              t.tile_elems, smem);
   FE_CUDA(cudaFuncSetAttribute(ebe_gather_kernel<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  ebe_gather_kernel<T, R><<<(unsigned)t.n_tiles, kThreads, smem, s>>>(
-      m->view<T>(), t.tile_elems, t.node_ptr.as<int32_t>(), t.node_ids.as<int32_t>(), t.node_own.as<uint8_t>(),
-      t.lconn.as<uint16_t>(), t.inc.as<uint16_t>(), t.inc_start.as<uint16_t>(), x, y, skip);
-  FE_CHECK_LAUNCH();
+  launch_behind_zero(ebe_gather_kernel<T, R>, t.n_tiles, kThreads, smem, s, m->view<T>(), t.tile_elems,
+                     t.node_ptr.as<int32_t>(), t.node_ids.as<int32_t>(), t.node_own.as<uint8_t>(),
+                     t.lconn.as<uint16_t>(), t.inc.as<uint16_t>(), t.inc_start.as<uint16_t>(), x, y, skip);
 }
 
 template <typename T, int R, int CPT = 1>
