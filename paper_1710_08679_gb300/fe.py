@@ -138,9 +138,15 @@ def version() -> str:
     return load().fe_version().decode()
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream_ptr(device):
@@ -211,7 +217,8 @@ class Mesh:
         return 3 * self.n_nodes
 
     def _stream(self):
-        return _stream_ptr(_torch().device("cuda", self.device))
+        # the raw handle: current_stream() builds a Stream object, 2.6 us of a 16 us small product
+        return _torch()._C._cuda_getCurrentRawStream(self.device)
 
     # ---- operator -------------------------------------------------------
     def ebe(self, x, out=None):
@@ -220,13 +227,19 @@ class Mesh:
         if x.dim() != 3 or x.shape[0] != self.n_nodes or x.shape[2] != 3:
             raise ValueError("x must be [N, R, 3]")
         R = int(x.shape[1])
-        dt = {torch.float64: FE_F64, torch.float32: FE_F32}.get(x.dtype)
+        dt = FE_F64 if x.dtype == torch.float64 else FE_F32 if x.dtype == torch.float32 else None
         if dt is None:
             raise TypeError("x must be float64 or float32")
         xp = _dev_ptr(x, x.dtype, name="x")
-        y = torch.empty_like(x) if out is None else out
-        yp = _dev_ptr(y, x.dtype, x.shape, name="out")
-        _check(load().fe_ebe_apply(self._h, R, dt, xp, yp, self._stream()), "fe_ebe_apply")
+        if out is None:
+            y = torch.empty_like(x)
+            yp = y.data_ptr()
+        else:
+            y = out
+            yp = _dev_ptr(y, x.dtype, x.shape, name="out")
+        st = load().fe_ebe_apply(self._h, R, dt, xp, yp, self._stream())
+        if st != FE_OK:
+            _check(st, "fe_ebe_apply")
         return y
 
     def ebe_host(self, x, out=None):
