@@ -1030,6 +1030,8 @@ __global__ void __launch_bounds__(PipeThreads<T, CPT>::value) ebe_pipe_kernel(in
 // phase 1 splits the gathered FP64 inputs in place (integer operations), and
 // phase 3 converts each node sum back to FP64 before its atomic add.
 // ---------------------------------------------------------------------------
+// Writes the layout of elem_apply_df_pair (corner pairs side by side, V/5 folded into the
+// Lame constants and a power of two).
 __global__ void __launch_bounds__(kThreads) prep_df_kernel(MeshView<double> M, df* __restrict__ geo, int64_t nv,
                                                            double* __restrict__ y, const int* __restrict__ skip) {
   if (skip && *skip) return;
@@ -1040,21 +1042,21 @@ __global__ void __launch_bounds__(kThreads) prep_df_kernel(MeshView<double> M, d
     load_conn<double>(M.conn, e, nd);
     ElemGeo<double> G;
     load_geometry(M, e, nd, G);
-    double v[kGeo];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-      for (int i = 0; i < 3; ++i) v[3 * k + i] = G.g[k][i];
-    v[12] = G.lam;
-    v[13] = G.mu;
-    v[14] = G.c;
-    v[15] = 0.0;
     float4* dst = reinterpret_cast<float4*>(geo + e * kGeo);
 #pragma unroll
-    for (int q = 0; q < kGeo / 2; ++q) {
-      const df a = df_split(v[2 * q]), b = df_split(v[2 * q + 1]);
-      dst[q] = make_float4(a.hi, a.lo, b.hi, b.lo);
-    }
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int P = 0; P < 2; ++P) {
+        const df a = df_split(G.g[2 * P][i]), b = df_split(G.g[2 * P + 1][i]);
+        dst[2 * i + P] = make_float4(a.hi, b.hi, a.lo, b.lo);
+      }
+    // V/5 = f 2^e, the exponent within float's range
+    const double c4 = 4.0 * G.c;
+    const int e2 = max(-126, min(126, (int)((__double_as_longlong(c4) >> 52) & 0x7FF) - 1023));
+    const double f = c4 * __longlong_as_double((long long)(1023 - e2) << 52);
+    const df a = df_split(G.lam * f), b = df_split(G.mu * f);
+    dst[6] = make_float4(a.hi, a.lo, b.hi, b.lo);
+    dst[7] = make_float4(0.f, 0.f, __int_as_float((e2 + 127) << 23), 0.f);
   }
   const int64_t n16 = nv / 2;
   for (int64_t i = gid; i < n16; i += stride) reinterpret_cast<double2*>(y)[i] = make_double2(0.0, 0.0);
@@ -1156,21 +1158,6 @@ __global__ void __launch_bounds__(kThreads) ebe_pipe_df_kernel(int64_t n_tiles, 
     for (int it = threadIdx.x; it < ne * R; it += blockDim.x) {
       const int le = it / R;
       const int r = it - le * R;
-      ElemGeo<df> Gm;
-      df gv[kGeo];
-#pragma unroll
-      for (int q = 0; q < kGeo / 2; ++q) {
-        const float4 w = reinterpret_cast<const float4*>(gs + le * kGeo)[q];
-        gv[2 * q] = df(w.x, w.y);
-        gv[2 * q + 1] = df(w.z, w.w);
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) Gm.g[k][d] = gv[3 * k + d];
-      Gm.lam = gv[12];
-      Gm.mu = gv[13];
-      Gm.c = gv[14];
       int off[12];
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
@@ -1180,20 +1167,7 @@ __global__ void __launch_bounds__(kThreads) ebe_pipe_df_kernel(int64_t n_tiles, 
         off[4 * q + 2] = w.z;
         off[4 * q + 3] = w.w;
       }
-      df u[10][3];
-#pragma unroll
-      for (int a = 0; a < 10; ++a) {
-        const df* xa = xcur + off[a] + 3 * r;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) u[a][c] = xa[c];
-      }
-      df yl[10][3];
-      elem_apply(Gm, u, yl);
-      df* o = ob + le * S + 3 * r;
-#pragma unroll
-      for (int a = 0; a < 10; ++a)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) o[a * VR + c] = yl[a][c];
+      elem_apply_df_pair<VR>(reinterpret_cast<const float4*>(gs + le * kGeo), xcur + 3 * r, off, ob + le * S + 3 * r);
     }
     __syncthreads();
 
@@ -1201,17 +1175,16 @@ __global__ void __launch_bounds__(kThreads) ebe_pipe_df_kernel(int64_t n_tiles, 
     for (int k = threadIdx.x; k < nn * CPN; k += blockDim.x) {
       const int ln = k / CPN;
       const int q = k - ln * CPN;
-      df a0, a1;
+      dfp a = {q_bc(0.f), q_bc(0.f)};
       const int j1 = is[ln + 1];
       const df* obq = ob + 2 * q;
       for (int j = is[ln]; j < j1; ++j) {
         const float4 w = *reinterpret_cast<const float4*>(obq + io[j]);
-        a0 += df(w.x, w.y);
-        a1 += df(w.z, w.w);
+        a = pnorm(padd(a, {make_float2(w.x, w.z), make_float2(w.y, w.w)}));
       }
       const int64_t gi = (int64_t)ids[ln] * VR + 2 * q;
       const int mk = mks[ln];
-      const df acc[2] = {a0, a1};
+      const df acc[2] = {df_two_sum(a.s.x, a.c.x), df_two_sum(a.s.y, a.c.y)};
 #pragma unroll
       for (int tt = 0; tt < 2; ++tt) {
         if ((mk >> ((2 * q + tt) % 3)) & 1)
@@ -1226,7 +1199,7 @@ __global__ void __launch_bounds__(kThreads) ebe_pipe_df_kernel(int64_t n_tiles, 
 // ---------------------------------------------------------------------------
 // Float-float kernel for two blocks per SM (FE_EBE_DF_LEAN). The tiles, packets,
 // split, slots and node sums of ebe_pipe_df_kernel, with
-//  * elem_apply_df_lean: node values and geometry read from shared memory where
+//  * elem_apply_df_pair: node values and geometry read from shared memory where
 //    they are used and outputs stored as they are formed, so the product fits in
 //    128 registers per thread; paired FP32 instructions over corners of the element
 //    (and over two values of a node in the sums);
@@ -1340,7 +1313,7 @@ __global__ void __launch_bounds__(kThreads, 2) ebe_pipe_df_lean_kernel(int64_t n
         off[4 * q + 2] = w.z;
         off[4 * q + 3] = w.w;
       }
-      elem_apply_df_lean<VR>(gs + le * kGeo, xcur + 3 * r, off, ob + le * S + 3 * r);
+      elem_apply_df_pair<VR>(reinterpret_cast<const float4*>(gs + le * kGeo), xcur + 3 * r, off, ob + le * S + 3 * r);
     }
     __syncthreads();
     // the next tile's rows into the one input buffer while the node sums run
@@ -1351,17 +1324,16 @@ __global__ void __launch_bounds__(kThreads, 2) ebe_pipe_df_lean_kernel(int64_t n
     for (int k = threadIdx.x; k < nn * CPN; k += blockDim.x) {
       const int ln = k / CPN;
       const int q = k - ln * CPN;
-      df a0, a1;
+      dfp a = {q_bc(0.f), q_bc(0.f)};
       const int j1 = is[ln + 1];
       const df* obq = ob + 2 * q;
       for (int j = is[ln]; j < j1; ++j) {
         const float4 w = *reinterpret_cast<const float4*>(obq + io[j]);
-        a0 += df(w.x, w.y);
-        a1 += df(w.z, w.w);
+        a = pnorm(padd(a, {make_float2(w.x, w.z), make_float2(w.y, w.w)}));
       }
       const int64_t gi = (int64_t)ids[ln] * VR + 2 * q;
       const int mk = mks[ln];
-      const df acc[2] = {a0, a1};
+      const df acc[2] = {df_two_sum(a.s.x, a.c.x), df_two_sum(a.s.y, a.c.y)};
 #pragma unroll
       for (int tt = 0; tt < 2; ++tt) {
         if ((mk >> ((2 * q + tt) % 3)) & 1)
