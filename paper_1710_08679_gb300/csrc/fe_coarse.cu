@@ -398,11 +398,38 @@ __global__ void __launch_bounds__(kThreads) spmv4_group_kernel(int64_t N4, int R
   o[2] = make_float4(acc[8], acc[9], acc[10], acc[11]);
 }
 
+// one block of the sliced matrix and the 4 cases' values of its column node
+struct SlicedTerm {
+  float m[9];
+  float4 v0, v1, v2;
+};
+__device__ __forceinline__ void load_x(SlicedTerm& t, const float* __restrict__ x, int64_t b, int R, int r0) {
+  const float4* xb = reinterpret_cast<const float4*>(x + (b * R + r0) * 3);
+  t.v0 = __ldg(xb);
+  t.v1 = __ldg(xb + 1);
+  t.v2 = __ldg(xb + 2);
+}
+__device__ __forceinline__ void load_m(SlicedTerm& t, const float* __restrict__ B) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k) t.m[k] = __ldg(B + 8 * k);
+}
+__device__ __forceinline__ void add_term(const SlicedTerm& t, float acc[12]) {
+  const float v[12] = {t.v0.x, t.v0.y, t.v0.z, t.v0.w, t.v1.x, t.v1.y, t.v1.z, t.v1.w, t.v2.x, t.v2.y, t.v2.z, t.v2.w};
+#pragma unroll
+  for (int w = 0; w < 4; ++w)
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      acc[3 * w + i] += t.m[3 * i] * v[3 * w] + t.m[3 * i + 1] * v[3 * w + 1] + t.m[3 * i + 2] * v[3 * w + 2];
+}
+
 // the same product from the sliced copy of the matrix: a warp's threads cover whole
 // 8-row slices, so each of the 9 value loads and the column load of a block reads
 // one sector for 8 rows (from the plain [nnzb][9] layout each read 8 sectors: ncu
-// showed the L1 88 % busy and 13 sectors per load request)
-__global__ void __launch_bounds__(kThreads) spmv4_sliced_kernel(int64_t N4, int R, const int32_t* __restrict__ rowptr,
+// showed the L1 88 % busy and 13 sectors per load request). The column and x are a
+// dependent pair of loads and the kernel waits on little else, so two blocks are in
+// flight at a time; 64 registers keep eight 128-thread CTAs on an SM (R = 16 on the 70x70x35
+// crust block: 57.4 -> 56.1 us).
+__global__ void __launch_bounds__(128, 8) spmv4_sliced_kernel(int64_t N4, int R, const int32_t* __restrict__ rowptr,
                                                                 const int32_t* __restrict__ sl_off,
                                                                 const int32_t* __restrict__ sl_cols,
                                                                 const float* __restrict__ sl_vals,
@@ -420,21 +447,24 @@ __global__ void __launch_bounds__(kThreads) spmv4_sliced_kernel(int64_t N4, int 
   float acc[12];
 #pragma unroll
   for (int i = 0; i < 12; ++i) acc[i] = 0.f;
-  for (int t = 0; t < len; ++t) {
-    const int64_t slot = base + t;
-    const int64_t b = __ldg(sl_cols + slot * 8 + rr);
-    const float* B = sl_vals + slot * 72 + rr;
-    float m[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) m[k] = __ldg(B + 8 * k);
-    const float4* xb = reinterpret_cast<const float4*>(x + (b * R + r0) * 3);
-    const float4 v0 = __ldg(xb), v1 = __ldg(xb + 1), v2 = __ldg(xb + 2);
-    const float v[12] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w, v2.x, v2.y, v2.z, v2.w};
-#pragma unroll
-    for (int w = 0; w < 4; ++w)
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-        acc[3 * w + i] += m[3 * i] * v[3 * w] + m[3 * i + 1] * v[3 * w + 1] + m[3 * i + 2] * v[3 * w + 2];
+  const int32_t* c = sl_cols + base * 8 + rr;
+  const float* B = sl_vals + base * 72 + rr;
+  int t = 0;
+  for (; t + 1 < len; t += 2, c += 16, B += 144) {
+    const int64_t b0 = __ldg(c), b1 = __ldg(c + 8);
+    SlicedTerm t0, t1;
+    load_x(t0, x, b0, R, r0);
+    load_x(t1, x, b1, R, r0);
+    load_m(t0, B);
+    load_m(t1, B + 72);
+    add_term(t0, acc);
+    add_term(t1, acc);
+  }
+  if (t < len) {
+    SlicedTerm t0;
+    load_x(t0, x, __ldg(c), R, r0);
+    load_m(t0, B);
+    add_term(t0, acc);
   }
   float4* o = reinterpret_cast<float4*>(y + (a * R + r0) * 3);
   o[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
@@ -755,7 +785,7 @@ void coarse_spmv(const fe_mesh* m, int R, const float* x4, float* y4, cudaStream
   const Coarse& c = m->coarse;
   FE_REQUIRE(c.csr_ready, "coarse matrix not assembled");
   if (R % 4 == 0 && c.sl_vals.ptr) {
-    spmv4_sliced_kernel<<<blocks_for(c.n_nodes * (R / 4)), kThreads, 0, s>>>(
+    spmv4_sliced_kernel<<<(unsigned)((c.n_nodes * (R / 4) + 127) / 128), 128, 0, s>>>(
         c.n_nodes, R, c.rowptr.as<int32_t>(), c.sl_off.as<int32_t>(), c.sl_cols.as<int32_t>(), c.sl_vals.as<float>(),
         x4, y4, skip);
     FE_CHECK_LAUNCH();
