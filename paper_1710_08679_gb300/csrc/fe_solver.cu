@@ -114,6 +114,23 @@ static VGeom vgeom(int64_t N, int R, int sms) {
   return g;
 }
 
+// the same for kernels with W cases per thread (R a multiple of W): blocks of K*G threads,
+// G = R/W, thread (j, g) handles node block*K + j and cases W g .. W g + W - 1 with 16-byte
+// loads. Reducing kernels: two blocks per SM, enough loads in flight, and fewer blocks do
+// less of the FP64 reduction at the end (an FP64 instruction takes as long as 61 others).
+static VGeom vgeom_w(int64_t N, int R, int W, int sms, int per_sm = 2) {
+  VGeom g;
+  g.R = R;
+  g.K = 1;
+  const int G = R / W;
+  while (g.K * 2 * G <= 256) g.K *= 2;
+  g.tpb = g.K * G;
+  const int64_t need = (N + g.K - 1) / g.K;
+  const int64_t cap = (int64_t)sms * per_sm;
+  g.grid = (unsigned)(need < cap ? need : cap);
+  return g;
+}
+
 // sums v over the K threads of each case in the block and adds the block total
 // to out[r] (FP64 atomics). Every thread of the block must call it.
 __device__ __forceinline__ void reduce_cases(double v, int R, int K, double* sm, double* out) {
@@ -126,6 +143,49 @@ __device__ __forceinline__ void reduce_cases(double v, int R, int K, double* sm,
   }
   if (j == 0) atomicAdd(out + threadIdx.x, sm[threadIdx.x]);
   __syncthreads();
+}
+
+// the same for NF fields and the W cases of each thread of a W-case kernel: field f's
+// totals go to out[f] + r. sm: [NF * W][blockDim.x] doubles.
+template <int NF, int W, typename T>
+__device__ __forceinline__ void reduce_cases_w(const T (&v)[NF][W], int G, double* sm, double* const (&out)[NF]) {
+  const int nt = blockDim.x;
+#pragma unroll
+  for (int f = 0; f < NF; ++f)
+#pragma unroll
+    for (int c = 0; c < W; ++c) sm[(W * f + c) * nt + threadIdx.x] = (double)v[f][c];
+  __syncthreads();
+  for (int w = nt >> 1; w >= G; w >>= 1) {   // nt = K G, K a power of two
+    for (int i = threadIdx.x; i < W * NF * w; i += nt) {
+      const int col = i / w, j = i - col * w;
+      sm[col * nt + j] += sm[col * nt + j + w];
+    }
+    __syncthreads();
+  }
+  for (int i = threadIdx.x; i < W * NF * G; i += nt) {
+    const int col = i / G, g = i - col * G;
+    atomicAdd(out[col / W] + W * g + col % W, sm[col * nt + g]);
+  }
+}
+
+__device__ __forceinline__ void load12(const float* p, float v[12]) {
+  const float4* q = reinterpret_cast<const float4*>(p);
+  const float4 a = q[0], b = q[1], c = q[2];
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+  v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  v[8] = c.x; v[9] = c.y; v[10] = c.z; v[11] = c.w;
+}
+
+__device__ __forceinline__ void store12(float* p, const float v[12]) {
+  float4* q = reinterpret_cast<float4*>(p);
+  q[0] = make_float4(v[0], v[1], v[2], v[3]);
+  q[1] = make_float4(v[4], v[5], v[6], v[7]);
+  q[2] = make_float4(v[8], v[9], v[10], v[11]);
+}
+
+__device__ __forceinline__ void load_block(const float* __restrict__ Bi, int64_t a, float m[9]) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k) m[k] = __ldg(Bi + 9 * a + k);
 }
 
 template <typename T>
@@ -465,14 +525,143 @@ __global__ void k_inner_update(int64_t N, Cases C, const float* __restrict__ Bi,
   reduce_cases((double)a2, C.R, blockDim.x / C.R, sm, C.d + D_RHOA * C.R);
 }
 
-// zq += ((double) ubar, q_prev)
-__global__ void k_outer_zq(int64_t N, Cases C, const float* __restrict__ ub, const double* __restrict__ q) {
+// The three passes of an inner step for R a multiple of 4: thread = (node, 4 cases), 48
+// contiguous bytes of each vector in three 16-byte loads and the node's block loaded once
+// for four cases. Same arithmetic per value as k_dot, k_inner_p and k_inner_update. Bound
+// by HBM at level 0 (R = 16, 1.41 M nodes: p, dot and update 0.56 -> 0.50 ms) and by L2 at
+// level 1 (0.086 -> 0.073 ms).
+#define GROUP_LOOP_BEGIN(W)                               \
+  const int R = C.R;                                      \
+  const int G = R / W;                                    \
+  const int r0 = W * (threadIdx.x % G);                   \
+  const int K = blockDim.x / G;                           \
+  const int64_t stride = (int64_t)gridDim.x * K;          \
+  for (int64_t n = (int64_t)blockIdx.x * K + threadIdx.x / G; n < N; n += stride) { \
+    const int64_t o = (n * R + r0) * 3;
+
+__global__ void __launch_bounds__(256) k_dot4(int64_t N, Cases C, int field, const int* __restrict__ skip,
+                                              const float* __restrict__ a, const float* __restrict__ b) {
   extern __shared__ double sm[];
-  double acc = 0.0;
-  VEC_LOOP_BEGIN
-  acc += (double)ub[o] * q[o] + (double)ub[o + 1] * q[o + 1] + (double)ub[o + 2] * q[o + 2];
+  if (skip && *skip) return;
+  float acc[1][4] = {};
+  GROUP_LOOP_BEGIN(4)
+  float x[12], y[12];
+  load12(a + o, x);
+  load12(b + o, y);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) acc[0][c] += x[3 * c] * y[3 * c] + x[3 * c + 1] * y[3 * c + 1] + x[3 * c + 2] * y[3 * c + 2];
   VEC_LOOP_END
-  reduce_cases(acc, C.R, blockDim.x / C.R, sm, C.d + D_ZQ * C.R);
+  reduce_cases_w<1, 4>(acc, C.R / 4, sm, {C.d + field * C.R});
+}
+
+__global__ void __launch_bounds__(256) k_inner_p4(int64_t N, Cases C, const float* __restrict__ Bi,
+                                                  const float* __restrict__ eb, float* __restrict__ pb) {
+  if (*C.done) return;
+  float be[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) be[c] = (float)C.D(D_BETAI, 4 * (threadIdx.x % (C.R / 4)) + c);
+  GROUP_LOOP_BEGIN(4)
+  float e[12], p[12], m[9];
+  load12(eb + o, e);
+  load12(pb + o, p);
+  load_block(Bi, n, m);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    float z[3];
+    mv3(m, e + 3 * c, z);
+    // the first step (beta = 0) must not use pbar: it holds the previous solve's data
+#pragma unroll
+    for (int k = 0; k < 3; ++k) p[3 * c + k] = be[c] != 0.f ? z[k] + be[c] * p[3 * c + k] : z[k];
+  }
+  store12(pb + o, p);
+  VEC_LOOP_END
+}
+
+__global__ void __launch_bounds__(256) k_inner_update4(int64_t N, Cases C, const float* __restrict__ Bi,
+                                                       float* __restrict__ eb, const float* __restrict__ qb,
+                                                       float* __restrict__ ub, const float* __restrict__ pb) {
+  extern __shared__ double sm[];
+  if (*C.done) return;
+  float al[4], acc[2][4] = {};
+#pragma unroll
+  for (int c = 0; c < 4; ++c) al[c] = (float)C.D(D_ALPHAI, 4 * (threadIdx.x % (C.R / 4)) + c);
+  GROUP_LOOP_BEGIN(4)
+  float e[12], q[12], u[12], p[12], m[9];
+  load12(eb + o, e);
+  load12(qb + o, q);
+  load12(ub + o, u);
+  load12(pb + o, p);
+  load_block(Bi, n, m);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    float z[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      e[3 * c + k] -= al[c] * q[3 * c + k];
+      u[3 * c + k] += al[c] * p[3 * c + k];
+    }
+    const float* v = e + 3 * c;
+    mv3(m, v, z);
+    acc[0][c] += v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+    acc[1][c] += z[0] * v[0] + z[1] * v[1] + z[2] * v[2];
+  }
+  store12(eb + o, e);
+  store12(ub + o, u);
+  VEC_LOOP_END
+  reduce_cases_w<2, 4>(acc, C.R / 4, sm, {C.d + D_EN2 * C.R, C.d + D_RHOA * C.R});
+}
+
+// float -> double by integer operations (a conversion instruction takes the FP64 pipe as
+// long as a multiply-add): exponent and mantissa moved into the double's fields. Subnormal,
+// infinite and NaN values take the conversion, in a function that is never inlined (see
+// fe_df.cuh).
+__device__ __noinline__ double widen_rare(float x) { return (double)x; }
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), e = b & 0x7f800000u, m = b & 0x7fffffffu;
+  if (e == 0x7f800000u || (e == 0u && m != 0u)) return widen_rare(x);
+  const unsigned hi = m == 0u ? b : (b & 0x80000000u) | ((m >> 3) + 0x38000000u);
+  return __hiloint2double((int)hi, (int)(b << 29));
+}
+
+__device__ __forceinline__ void load6(const double* p, double v[6]) {
+  const double2* q = reinterpret_cast<const double2*>(p);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const double2 a = q[k];
+    v[2 * k] = a.x;
+    v[2 * k + 1] = a.y;
+  }
+}
+__device__ __forceinline__ void load6(const float* p, double v[6]) {
+  const float2* q = reinterpret_cast<const float2*>(p);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float2 a = q[k];
+    v[2 * k] = widen(a.x);
+    v[2 * k + 1] = widen(a.y);
+  }
+}
+__device__ __forceinline__ void store6(double* p, const double v[6]) {
+  double2* q = reinterpret_cast<double2*>(p);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) q[k] = make_double2(v[2 * k], v[2 * k + 1]);
+}
+
+// zq += ((double) ubar, q_prev) ; rho += ((double) ubar, r), Algorithm 1(a)
+__global__ void k_outer_zq(int64_t N, Cases C, const float* __restrict__ ub, const double* __restrict__ q,
+                           const double* __restrict__ rv) {
+  extern __shared__ double sm[];
+  double a1 = 0.0, a2 = 0.0;
+  VEC_LOOP_BEGIN
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const double z = widen(ub[o + c]);
+    a1 += z * q[o + c];
+    a2 += z * rv[o + c];
+  }
+  VEC_LOOP_END
+  reduce_cases(a1, C.R, blockDim.x / C.R, sm, C.d + D_ZQ * C.R);
+  reduce_cases(a2, C.R, blockDim.x / C.R, sm, C.d + D_RHO * C.R);
 }
 
 // Algorithm 1(a), search direction: p = z + beta p with z = (double) ubar
@@ -481,26 +670,11 @@ __global__ void k_outer_p(int64_t N, Cases C, const float* __restrict__ ub, doub
   if (C.I(I_ACTIVE, r)) {
     const double be = C.D(D_BETA, r);
     if (be != 0.0)
-      for (int c = 0; c < 3; ++c) p[o + c] = (double)ub[o + c] + be * p[o + c];
+      for (int c = 0; c < 3; ++c) p[o + c] = widen(ub[o + c]) + be * p[o + c];
     else
-      for (int c = 0; c < 3; ++c) p[o + c] = (double)ub[o + c];
+      for (int c = 0; c < 3; ++c) p[o + c] = widen(ub[o + c]);
   }
   VEC_LOOP_END
-}
-
-// Algorithm 1(a): rho += (z, r) ; gam += (p, q)
-__global__ void k_outer_dots(int64_t N, Cases C, const float* __restrict__ ub, const double* __restrict__ rv,
-                             const double* __restrict__ p, const double* __restrict__ q) {
-  extern __shared__ double sm[];
-  double a1 = 0.0, a2 = 0.0;
-  VEC_LOOP_BEGIN
-  for (int c = 0; c < 3; ++c) {
-    a1 += (double)ub[o + c] * rv[o + c];
-    a2 += p[o + c] * q[o + c];
-  }
-  VEC_LOOP_END
-  reduce_cases(a1, C.R, blockDim.x / C.R, sm, C.d + D_RHO * C.R);
-  reduce_cases(a2, C.R, blockDim.x / C.R, sm, C.d + D_GAM * C.R);
 }
 
 // Algorithm 1(a), update: r -= alpha q ; u += alpha p ; rn2 += ||r||^2
@@ -520,6 +694,127 @@ __global__ void k_outer_update(int64_t N, Cases C, double* __restrict__ rv, cons
   }
   VEC_LOOP_END
   reduce_cases(acc, C.R, blockDim.x / C.R, sm, C.d + D_RN2 * C.R);
+}
+
+// The FP64 passes of an outer iteration for even R: thread = (node, 2 cases), 48 contiguous
+// bytes of an FP64 vector in three 16-byte loads. Same arithmetic per value as k_outer_zq,
+// k_outer_p, k_dot, k_outer_update and k_cast_start. Bound by HBM once the FP64 pipe has
+// only the multiply-adds to do (R = 16, 1.41 M nodes, with the conversions there and 8-byte
+// loads: 0.30, 0.30, 0.38, 0.66 and 0.25 ms; (z, r) then needed z a second time).
+__global__ void __launch_bounds__(256) k_outer_zq2(int64_t N, Cases C, const float* __restrict__ ub,
+                                                   const double* __restrict__ q, const double* __restrict__ rv) {
+  extern __shared__ double sm[];
+  double acc[2][2] = {};
+  GROUP_LOOP_BEGIN(2)
+  double z[6], a[6], b[6];
+  load6(ub + o, z);
+  load6(q + o, a);
+  load6(rv + o, b);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    acc[0][k / 3] += z[k] * a[k];
+    acc[1][k / 3] += z[k] * b[k];
+  }
+  VEC_LOOP_END
+  reduce_cases_w<2, 2>(acc, C.R / 2, sm, {C.d + D_ZQ * C.R, C.d + D_RHO * C.R});
+}
+
+__global__ void __launch_bounds__(256) k_dot_f64_2(int64_t N, Cases C, int field, const double* __restrict__ a,
+                                                   const double* __restrict__ b) {
+  extern __shared__ double sm[];
+  double acc[1][2] = {};
+  GROUP_LOOP_BEGIN(2)
+  double x[6], y[6];
+  load6(a + o, x);
+  load6(b + o, y);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) acc[0][k / 3] += x[k] * y[k];
+  VEC_LOOP_END
+  reduce_cases_w<1, 2>(acc, C.R / 2, sm, {C.d + field * C.R});
+}
+
+__global__ void __launch_bounds__(256) k_outer_p2(int64_t N, Cases C, const float* __restrict__ ub,
+                                                  double* __restrict__ p) {
+  double be[2];
+  bool act[2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const int r = 2 * (threadIdx.x % (C.R / 2)) + c;
+    act[c] = C.I(I_ACTIVE, r);
+    be[c] = C.D(D_BETA, r);
+  }
+  if (!act[0] && !act[1]) return;
+  GROUP_LOOP_BEGIN(2)
+  double z[6], v[6];
+  load6(ub + o, z);
+  load6(p + o, v);
+#pragma unroll
+  for (int k = 0; k < 6; ++k)
+    if (act[k / 3]) v[k] = be[k / 3] != 0.0 ? z[k] + be[k / 3] * v[k] : z[k];
+  store6(p + o, v);
+  VEC_LOOP_END
+}
+
+__global__ void __launch_bounds__(256) k_outer_update2(int64_t N, Cases C, double* __restrict__ rv,
+                                                       const double* __restrict__ q, double* __restrict__ u,
+                                                       const double* __restrict__ p) {
+  extern __shared__ double sm[];
+  double al[2], acc[1][2] = {};
+  bool act[2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const int r = 2 * (threadIdx.x % (C.R / 2)) + c;
+    act[c] = C.I(I_ACTIVE, r);
+    al[c] = C.D(D_ALPHA, r);
+  }
+  if (act[0] || act[1]) {
+    GROUP_LOOP_BEGIN(2)
+    double a[6], b[6], x[6], y[6];
+    load6(rv + o, a);
+    load6(q + o, b);
+    load6(u + o, x);
+    load6(p + o, y);
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+      if (act[k / 3]) {
+        a[k] -= al[k / 3] * b[k];
+        x[k] += al[k / 3] * y[k];
+        acc[0][k / 3] += a[k] * a[k];
+      }
+    store6(rv + o, a);
+    store6(u + o, x);
+    VEC_LOOP_END
+  }
+  reduce_cases_w<1, 2>(acc, C.R / 2, sm, {C.d + D_RN2 * C.R});
+}
+
+__global__ void __launch_bounds__(256) k_cast_start2(int64_t N, Cases C, const float* __restrict__ Bi,
+                                                     const double* __restrict__ rv, float* __restrict__ rb,
+                                                     float* __restrict__ ub) {
+  extern __shared__ double sm[];
+  float acc[1][2] = {};
+  bool act[2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) act[c] = C.I(I_ACTIVE, 2 * (threadIdx.x % (C.R / 2)) + c);
+  GROUP_LOOP_BEGIN(2)
+  double d[6];
+  float v[6], z[6], m[9];
+  load6(rv + o, d);
+  load_block(Bi, n, m);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) v[k] = act[k / 3] ? (float)d[k] : 0.f;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    mv3(m, v + 3 * c, z + 3 * c);
+    acc[0][c] += v[3 * c] * v[3 * c] + v[3 * c + 1] * v[3 * c + 1] + v[3 * c + 2] * v[3 * c + 2];
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    reinterpret_cast<float2*>(rb + o)[k] = make_float2(v[2 * k], v[2 * k + 1]);
+    reinterpret_cast<float2*>(ub + o)[k] = make_float2(z[2 * k], z[2 * k + 1]);
+  }
+  VEC_LOOP_END
+  reduce_cases_w<1, 2>(acc, C.R / 2, sm, {C.d + D_RBN2 * C.R});
 }
 
 // true residuals of the candidate cases from one all-case product t = K u:
@@ -754,6 +1049,7 @@ __global__ void s_outer_begin(Cases C) {
   C.D(D_EN2, r) = 0.0;
   C.D(D_RHOA, r) = 0.0;
   C.D(D_ZQ, r) = 0.0;
+  C.D(D_RHO, r) = 0.0;
   if (r == 0) {
     *C.done = 0;
     C.step() = 0;
@@ -831,7 +1127,6 @@ __global__ void s_outer_beta(Cases C, int literal) {
     C.I(I_RESTART, r) = 0;
   }
   C.D(D_BETA, r) = be;
-  C.D(D_RHO, r) = 0.0;
   C.D(D_GAM, r) = 0.0;
 }
 
@@ -991,26 +1286,6 @@ __device__ __forceinline__ void row_times(const InnerArgs& A, int64_t a, int r0,
       for (int i = 0; i < 3; ++i)
         acc[3 * w + i] += m[3 * i] * v[3 * w] + m[3 * i + 1] * v[3 * w + 1] + m[3 * i + 2] * v[3 * w + 2];
   }
-}
-
-__device__ __forceinline__ void load12(const float* p, float v[12]) {
-  const float4* q = reinterpret_cast<const float4*>(p);
-  const float4 a = q[0], b = q[1], c = q[2];
-  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-  v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-  v[8] = c.x; v[9] = c.y; v[10] = c.z; v[11] = c.w;
-}
-
-__device__ __forceinline__ void store12(float* p, const float v[12]) {
-  float4* q = reinterpret_cast<float4*>(p);
-  q[0] = make_float4(v[0], v[1], v[2], v[3]);
-  q[1] = make_float4(v[4], v[5], v[6], v[7]);
-  q[2] = make_float4(v[8], v[9], v[10], v[11]);
-}
-
-__device__ __forceinline__ void load_block(const float* __restrict__ Bi, int64_t a, float m[9]) {
-#pragma unroll
-  for (int k = 0; k < 9; ++k) m[k] = __ldg(Bi + 9 * a + k);
 }
 
 // adds a thread's 4-case partial sums (FP32, widened) of NF consecutive fields
@@ -1221,6 +1496,7 @@ struct Solve {
   VGeom g1;
   int64_t N2 = 0;  // level-2 aggregates (0: no level 2)
   VGeom g2;
+  int sms = 0;
   bool assembled1 = false;  // level-1 operator: assembled block CSR, else element by element
   cudaStream_t s;
   const double* f;
@@ -1230,6 +1506,13 @@ struct Solve {
   template <typename K, typename... A>
   void vec(K kern, A... args) {
     kern<<<g.grid, g.tpb, sm, s>>>(N, C, args...);
+    FE_CHECK_LAUNCH();
+  }
+  // a kernel with two cases per thread (R even) reducing `nf` fields
+  template <typename K, typename... A>
+  void vec_w(K kern, int nf, A... args) {
+    const VGeom g2 = vgeom_w(N, R, 2, sms, nf > 0 ? 3 : 8);
+    kern<<<g2.grid, g2.tpb, 2 * (size_t)nf * g2.tpb * sizeof(double), s>>>(N, C, args...);
     FE_CHECK_LAUNCH();
   }
   // the same vector kernel over `n` nodes with launch geometry `gg` (level 1)
@@ -1337,6 +1620,20 @@ static void level_apply(Solve& S, const Level& L, const float* x, float* y, cons
 
 // one inner step (Algorithm 1(b)) and the stop test for the next one
 static void inner_step(Solve& S, const Level& L, cudaGraphConditionalHandle loop, int use_loop) {
+  if (S.R % 4 == 0) {
+    const VGeom g4 = vgeom_w(L.N, S.R, 4, S.sms), gp = vgeom_w(L.N, S.R, 4, S.sms, 6);
+    const size_t col = 4 * (size_t)g4.tpb * sizeof(double);
+    k_inner_p4<<<gp.grid, gp.tpb, 0, S.s>>>(L.N, S.C, L.B, L.eb, L.pb);
+    FE_CHECK_LAUNCH();
+    level_apply(S, L, L.pb, L.qb, S.C.done);
+    k_dot4<<<g4.grid, g4.tpb, col, S.s>>>(L.N, S.C, (int)D_GAMI, S.C.done, L.pb, L.qb);
+    FE_CHECK_LAUNCH();
+    S.scal(s_inner_alpha, L.f_rbn2, L.f_count);
+    k_inner_update4<<<g4.grid, g4.tpb, 2 * col, S.s>>>(L.N, S.C, L.B, L.eb, L.qb, L.ub, L.pb);
+    FE_CHECK_LAUNCH();
+    S.scal(s_inner_check, L.n, L.eps, L.f_rbn2, loop, use_loop);
+    return;
+  }
   S.vec_on(L.N, *L.g, k_inner_p, L.B, (const float*)L.eb, L.pb);
   level_apply(S, L, L.pb, L.qb, S.C.done);
   S.vec_on(L.N, *L.g, k_dot<float>, (int)D_GAMI, (const int*)S.C.done, (const float*)L.pb, (const float*)L.qb);
@@ -1489,7 +1786,9 @@ static void fcg_iteration(Solve& S) {
   fe_mesh* m = S.m;
   const float* B32 = m->binv32.as<float>();
   S.scal(s_outer_begin);
-  S.vec(k_cast_start, B32, w->r.as<double>(), w->rb.as<float>(), w->ub.as<float>());
+  const bool even = S.R % 2 == 0;   // two cases per thread
+  if (even) S.vec_w(k_cast_start2, 1, B32, w->r.as<double>(), w->rb.as<float>(), w->ub.as<float>());
+  else S.vec(k_cast_start, B32, w->r.as<double>(), w->rb.as<float>(), w->ub.as<float>());
   if (S.N1 > 0) {
     Level L1{S.N1, &S.g1, m->coarse.binv32.as<float>(), w->rb1.as<float>(), w->ub1.as<float>(),
              w->eb1.as<float>(), w->pb1.as<float>(), w->qb1.as<float>(), 1, S.o.n_inner1, S.o.eps_inner1,
@@ -1517,14 +1816,21 @@ static void fcg_iteration(Solve& S) {
   Level L0{S.N, &S.g, B32, w->rb.as<float>(), w->ub.as<float>(), w->eb.as<float>(), w->pb.as<float>(),
            w->qb.as<float>(), 0, S.o.n_inner, S.o.eps_inner, (int)D_RBN2, (int)I_INNER};
   inner_loop(S, L0);
-  S.vec(k_outer_zq, (const float*)w->ub.as<float>(), (const double*)w->q.as<double>());
+  const float* ub = w->ub.as<float>();
+  const double *pc = w->p.as<double>(), *q = w->q.as<double>(), *rc = w->r.as<double>();
+  if (even) S.vec_w(k_outer_zq2, 2, ub, q, rc);
+  else S.vec(k_outer_zq, ub, q, rc);
   S.scal(s_outer_beta, S.o.literal_beta);
-  S.vec(k_outer_p, (const float*)w->ub.as<float>(), w->p.as<double>());
-  ebe_apply<double>(m, S.R, w->p.as<double>(), w->q.as<double>(), S.s);
-  S.vec(k_outer_dots, (const float*)w->ub.as<float>(), (const double*)w->r.as<double>(),
-        (const double*)w->p.as<double>(), (const double*)w->q.as<double>());
+  if (even) S.vec_w(k_outer_p2, 0, ub, w->p.as<double>());
+  else S.vec(k_outer_p, ub, w->p.as<double>());
+  ebe_apply<double>(m, S.R, pc, w->q.as<double>(), S.s);
+  if (even) S.vec_w(k_dot_f64_2, 1, (int)D_GAM, pc, q);
+  else S.vec(k_dot<double>, (int)D_GAM, (const int*)nullptr, pc, q);
   S.scal(s_outer_alpha);
-  S.vec(k_outer_update, w->r.as<double>(), (const double*)w->q.as<double>(), S.u, (const double*)w->p.as<double>());
+  if (even && ((uintptr_t)S.u & 15) == 0)   // the caller's u has no alignment rule
+    S.vec_w(k_outer_update2, 1, w->r.as<double>(), q, S.u, pc);
+  else
+    S.vec(k_outer_update, w->r.as<double>(), q, S.u, pc);
   S.scal(s_outer_check, S.o.tol, S.o.max_outer);
 }
 
@@ -1587,6 +1893,7 @@ static fe_status run_solve(fe_mesh* m, int R, const double* f, double* u, const 
     S.C.hist = hist.as<double>();
     S.C.hist_len = o.cg_coef_len;
   }
+  S.sms = sms;
   S.g = vgeom(S.N, R, sms);
   S.sm = (size_t)S.g.tpb * sizeof(double);
   S.s = s;

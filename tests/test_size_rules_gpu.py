@@ -82,6 +82,38 @@ def test_warp_specialised_product(case, R, variant, tile):
         assert rel_l2(y[:, r], ref[:, r]) <= TOL32, r
 
 
+# R = 12, 20: groups of 4 cases whose number is no power of two; 5 and 6: the one- and
+# two-case passes; 32: the largest. `shift`: u on an 8-byte boundary only.
+@pytest.mark.gpu
+@pytest.mark.parametrize("R,shift", [(4, 0), (5, 0), (6, 0), (6, 1), (12, 0), (20, 0), (32, 0)])
+@pytest.mark.parametrize("solver", ["fcg_mixed", "fcg_mg"])
+def test_inner_and_outer_passes(solver, R, shift):
+    ensure_lib()
+    import ctypes
+
+    from paper_1710_08679_gb300 import fe
+    m = MESHES["ragged"]()
+    K = oracle.assemble(m)
+    f = mg.random_vectors(m.n_nodes, R, seed=7) * m.free[:, None, :]
+    f[:, R - 1] = 0.0   # a case that is finished at the start
+    M = fe.Mesh.from_mesh(m)
+    F = cuda(f)
+    u = torch.zeros(F.numel() + shift, dtype=torch.float64, device="cuda")[shift:]
+    o = fe.SolveOpts()
+    fe.load().fe_solve_opts_default(ctypes.byref(o))
+    o.solver, o.tol = fe.SOLVERS[solver], 1e-8
+    stats = (fe.SolveStats * R)()
+    torch.cuda.synchronize()
+    st = fe.load().fe_pcg_solve(M.handle, R, F.data_ptr(), u.data_ptr(), ctypes.byref(o), stats, None)
+    torch.cuda.synchronize()
+    assert st == fe.FE_OK
+    u = u.view(F.shape).cpu().numpy()
+    ref = oracle.direct_solve(K, f)
+    for r in range(R - 1):
+        assert stats[r].relres <= 1e-8 and rel_l2(u[:, r], ref[:, r]) <= 1e-6, r
+    assert not np.any(u[:, R - 1])
+
+
 # cases that converge one after the other leave and re-enter the device-side loop
 @pytest.mark.gpu
 @pytest.mark.parametrize("R", [1, 3, 6])
