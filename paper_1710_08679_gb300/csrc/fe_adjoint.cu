@@ -53,7 +53,7 @@ __device__ __forceinline__ void strain_energy(const double e[6], const double f[
 // with lam and mu applied after the sum over the cases: about 450 instructions per case,
 // where forming K_e u_e and its product with lambda_e took about 490. One-warp blocks and
 // the split (f64_case_split) even out the last round. 16 cases on the 82,944 elements of the
-// 24^3 box: 1421 -> 1307 us; error against 64-bit torch 4.06e-16 (before 4.36e-16).
+// 24^3 box: 1418 -> 1296 us; error against 64-bit torch 4.06e-16 (before 4.36e-16).
 __global__ void __launch_bounds__(32) adjoint_kernel(MeshView<double> M, int R, int split,
                                                      const int64_t* __restrict__ perm, const double* __restrict__ u,
                                                      const double* __restrict__ lam, double* __restrict__ g) {
@@ -76,7 +76,9 @@ __global__ void __launch_bounds__(32) adjoint_kernel(MeshView<double> M, int R, 
 #pragma unroll
     for (int i = 0; i < 3; ++i) xc[k][i] = __ldg(M.xyz + 3 * (int64_t)nd[k] + i);
   ElemGeo<double> G;
-  elem_geometry(xc[0], xc[1], xc[2], xc[3], __ldg(M.mat + 2 * e), __ldg(M.mat + 2 * e + 1), G);
+  elem_gradients(xc[0], xc[1], xc[2], xc[3], G);
+  G.lam = __ldg(M.lame + 2 * e);
+  G.mu = __ldg(M.lame + 2 * e + 1);
   double g3[4][3];
 #pragma unroll
   for (int k = 0; k < 4; ++k)

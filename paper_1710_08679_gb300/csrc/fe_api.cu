@@ -8,6 +8,7 @@
 #include <string>
 #include <vector>
 
+#include "fe_element.cuh"
 #include "fe_internal.cuh"
 
 namespace fe {
@@ -272,6 +273,14 @@ void build_colouring(fe_mesh* m, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // materials upload (internal element order)
 // ---------------------------------------------------------------------------
+__global__ void lame_kernel(int64_t E, const double2* __restrict__ mat, double2* __restrict__ lame) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= E) return;
+  double2 v;
+  fe::lame_constants(mat[e].x, mat[e].y, v.x, v.y);
+  lame[e] = v;
+}
+
 static void upload_materials(fe_mesh* m, cudaStream_t s) {
   const int64_t E = m->n_elem;
   std::vector<double> m64((size_t)E * 2);
@@ -291,6 +300,8 @@ static void upload_materials(fe_mesh* m, cudaStream_t s) {
   FE_CUDA(cudaMemcpyAsync(m->mat64.ptr, m64.data(), m64.size() * 8, cudaMemcpyHostToDevice, s));
   FE_CUDA(cudaMemcpyAsync(m->mat32.ptr, m32.data(), m32.size() * 4, cudaMemcpyHostToDevice, s));
   FE_CUDA(cudaMemcpyAsync(m->matv.ptr, mv.data(), mv.size() * 4, cudaMemcpyHostToDevice, s));
+  lame_kernel<<<(unsigned)((E + 255) / 256), 256, 0, s>>>(E, m->mat64.as<double2>(), m->lame64.as<double2>());
+  FE_CHECK_LAUNCH();
   fe::ws_refresh_materials(m, s);
   FE_CUDA(cudaStreamSynchronize(s));
   m->jacobi_ready = false;
@@ -304,11 +315,11 @@ static void upload_materials(fe_mesh* m, cudaStream_t s) {
 
 template <>
 fe::MeshView<double> fe_mesh::view<double>() const {
-  return {n_nodes, n_elem, conn.as<int32_t>(), xyz64.as<double>(), mat64.as<double>(), nmask.as<uint8_t>()};
+  return {n_nodes, n_elem, conn.as<int32_t>(), xyz64.as<double>(), mat64.as<double>(), nmask.as<uint8_t>(), lame64.as<double>()};
 }
 template <>
 fe::MeshView<float> fe_mesh::view<float>() const {
-  return {n_nodes, n_elem, conn.as<int32_t>(), xyz32.as<float>(), mat32.as<float>(), nmask.as<uint8_t>()};
+  return {n_nodes, n_elem, conn.as<int32_t>(), xyz32.as<float>(), mat32.as<float>(), nmask.as<uint8_t>(), nullptr};
 }
 
 using namespace fe;
@@ -413,6 +424,7 @@ fe_status fe_mesh_create(int64_t n_nodes, const double* coords, int64_t n_elem, 
     m->xyz64.alloc((size_t)n_nodes * 3 * sizeof(double));
     m->xyz32.alloc((size_t)n_nodes * 3 * sizeof(float));
     m->mat64.alloc((size_t)n_elem * 2 * sizeof(double));
+    m->lame64.alloc((size_t)n_elem * 2 * sizeof(double));
     m->mat32.alloc((size_t)n_elem * 2 * sizeof(float));
     m->matv.alloc((size_t)n_elem * 4 * sizeof(float));
     m->dev_status.alloc(sizeof(int32_t));

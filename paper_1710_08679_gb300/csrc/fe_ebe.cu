@@ -80,7 +80,13 @@ __device__ __forceinline__ void load_geometry(const MeshView<T>& M, int64_t e, c
   for (int k = 0; k < 4; ++k)
 #pragma unroll
     for (int i = 0; i < 3; ++i) xc[k][i] = __ldg(M.xyz + 3 * (int64_t)nd[k] + i);
-  elem_geometry(xc[0], xc[1], xc[2], xc[3], __ldg(M.mat + 2 * e), __ldg(M.mat + 2 * e + 1), G);
+  if constexpr (sizeof(T) == 8) {
+    elem_gradients(xc[0], xc[1], xc[2], xc[3], G);
+    G.lam = __ldg(M.lame + 2 * e);
+    G.mu = __ldg(M.lame + 2 * e + 1);
+  } else {
+    elem_geometry(xc[0], xc[1], xc[2], xc[3], __ldg(M.mat + 2 * e), __ldg(M.mat + 2 * e + 1), G);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -134,7 +140,9 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) ebe_direct_kern
 // FP64 direct kernel: thread = (element, share of the cases); lane `part` of an
 // element's `split` lanes takes cases part, part + split, ... Bound by the FP64 pipe (1/61
 // of FP32), so the geometry, a fifth of a case's FP64 instructions, is computed once
-// per thread, and blocks of one warp fill the SMs evenly.
+// per thread, and blocks of one warp fill the SMs evenly. 5 cases on the 146,124 elements of
+// the 41x33x18 crust block: 812 -> 678 us; one case on the 1.03 M elements of the 70x70x35
+// block: 1142 -> 980 us (0.92 TFLOP/s of 1.2), 50 us of it from the stored Lame constants.
 __global__ void __launch_bounds__(32) ebe_direct_f64_kernel(MeshView<double> M, int R, int split,
                                                             const uint16_t* __restrict__ own,
                                                             const double* __restrict__ x, double* __restrict__ y,
@@ -179,11 +187,11 @@ __global__ void __launch_bounds__(32) ebe_direct_f64_kernel(MeshView<double> M, 
 // FP64 direct kernel for few items: four lanes per (element, case), lane m = corner m. A
 // warp's FP64 instruction occupies its SM sub-partition for some 60 cycles whatever the
 // other sub-partitions do, so with fewer warps than sub-partitions (608) the time is one
-// warp's FP64 instruction count: 588 with a lane per element. Here a lane forms its
-// corner's gradient (one of the three quotients 1/det, lam, mu per lane), stress s_m,
-// corner output and its terms T_m g_l of the three edges at its corner: about 200. One case
-// on the 3,072 elements of the 8^3 box: 25 us with a lane per element (kernel); the whole
-// product 28.3 (gather kernel, the fastest before) -> 18.1 us; a 172-step PCG solve 7.6 -> 5.1 ms.
+// warp's FP64 instruction count: about 550 with a lane per element. Here a lane forms its
+// corner's gradient, stress s_m, corner output and its terms T_m g_l of the three edges at
+// its corner: about 185. One case on the 3,072 elements of the 8^3 box: 25 us with a lane per
+// element (kernel); the whole product 28.3 (gather kernel, the fastest before) -> 18.1 us; a
+// 172-step PCG solve 7.6 -> 5.1 ms.
 __global__ void __launch_bounds__(64) ebe_corner_f64_kernel(MeshView<double> M, int R,
                                                             const uint16_t* __restrict__ own,
                                                             const double* __restrict__ x, double* __restrict__ y,
@@ -236,14 +244,9 @@ __global__ void __launch_bounds__(64) ebe_corner_f64_kernel(MeshView<double> M, 
   n[2] = d2[0] * d3[1] - d2[1] * d3[0];
   const double dets = dm[0] * n[0] + dm[1] * n[1] + dm[2] * n[2];
   const double det = fabs(dets);
-  const double E = __ldg(M.mat + 2 * e), nu = __ldg(M.mat + 2 * e + 1), onu = 1.0 + nu;
-  // lanes 0, 1: mu, lam; lanes 2, 3: the reciprocal determinant
-  const double num = m == 0 ? E : m == 1 ? E * nu : 1.0;
-  const double den = m == 0 ? 2.0 * onu : m == 1 ? onu * (1.0 - 2.0 * nu) : det;
-  const double quo = num / den;
-  const double c4 = __shfl_sync(kAll, det, 0, 4) * (1.0 / 30.0);   // V/5
-  const double mu = __shfl_sync(kAll, quo, 0, 4) * c4, lam = __shfl_sync(kAll, quo, 1, 4) * c4;
-  double inv = __shfl_sync(kAll, quo, 2, 4);
+  const double c4 = det * (1.0 / 30.0);   // V/5
+  const double lam = __ldg(M.lame + 2 * e) * c4, mu = __ldg(M.lame + 2 * e + 1) * c4;
+  double inv = 1.0 / det;
   if (dets < 0.0) inv = -inv;
   double g[4][3];   // g of corners m, m + 1, m + 2, m + 3
 #pragma unroll
@@ -1383,7 +1386,7 @@ static void launch_direct(const fe_mesh* m, int R, const T* x, T* y, cudaStream_
     int64_t cost = 0;
     const int split = f64_case_split(M.n_elem, R, 438, sms, &cost);
     const int64_t lanes = 4 * M.n_elem * R, units = 4 * (int64_t)sms;
-    if (((lanes + 31) / 32 + units - 1) / units * 200 < cost) {
+    if (((lanes + 31) / 32 + units - 1) / units * 185 < cost) {
       launch_behind_zero(ebe_corner_f64_kernel, (lanes + 63) / 64, 64, 0, s, M, R, m->own_elem.as<uint16_t>(), x, y, skip);
       return;
     }

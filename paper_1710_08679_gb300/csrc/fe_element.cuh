@@ -48,11 +48,10 @@ struct ElemGeo {
   T c;        // element volume / 20
 };
 
-// Geometry and Lame constants of one element from its corner coordinates.
-// Returns 6V (positive for a valid element).
+// Gradients and volume of one element from its corner coordinates. Returns 6V (positive
+// for a valid element).
 template <typename T>
-__device__ __forceinline__ T elem_geometry(const T x0[3], const T x1[3], const T x2[3], const T x3[3],
-                                           T E, T nu, ElemGeo<T>& G) {
+__device__ __forceinline__ T elem_gradients(const T x0[3], const T x1[3], const T x2[3], const T x3[3], ElemGeo<T>& G) {
   T d1[3], d2[3], d3[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -74,10 +73,22 @@ __device__ __forceinline__ T elem_geometry(const T x0[3], const T x1[3], const T
     G.g[0][i] = -(G.g[1][i] + G.g[2][i] + G.g[3][i]);
   }
   G.c = det * T(1.0 / 120.0);
-  T onu = T(1) + nu;
-  G.mu = E / (T(2) * onu);
-  G.lam = (E * nu) / (onu * (T(1) - T(2) * nu));
   return det;
+}
+
+template <typename T>
+__device__ __forceinline__ void lame_constants(T E, T nu, T& lam, T& mu) {
+  const T onu = T(1) + nu;
+  mu = E / (T(2) * onu);
+  lam = (E * nu) / (onu * (T(1) - T(2) * nu));
+}
+
+// Geometry and Lame constants of one element
+template <typename T>
+__device__ __forceinline__ T elem_geometry(const T x0[3], const T x1[3], const T x2[3], const T x3[3],
+                                           T E, T nu, ElemGeo<T>& G) {
+  lame_constants(E, nu, G.lam, G.mu);
+  return elem_gradients(x0, x1, x2, x3, G);
 }
 
 // w = s g for a symmetric 3x3 s stored (xx, yy, zz, yz, xz, xy)

@@ -94,6 +94,8 @@ struct MeshView {
   const T* xyz;          // [N][3]
   const T* mat;          // [E][2]  (E, nu)
   const uint8_t* nmask;  // [N]     bit c set <=> DOF c of the node is free
+  const T* lame;         // [E][2]  (lam, mu), FP64 only: two divisions are a quarter of the FP64
+                         //         instructions of an element's geometry
 };
 
 // Tiles of elements for the shared-memory accumulation kernel.
@@ -224,6 +226,7 @@ struct fe_mesh {
   fe::DevBuf xyz64;     // double [N][3]
   fe::DevBuf xyz32;     // float [N][3]
   fe::DevBuf mat64;     // double [E][2]
+  fe::DevBuf lame64;    // double [E][2] lam, mu of the materials in mat64 (refreshed with them)
   fe::DevBuf mat32;     // float [E][2]
   fe::DevBuf nmask;     // uint8 [N]
   std::vector<double> young_host;
@@ -312,14 +315,14 @@ void build_block_jacobi(fe_mesh* m, cudaStream_t s);
 // cases (a power of two at most 32). Each SM sub-partition runs its share of the warps
 // through its FP64 unit one instruction after the other, so the time is the largest
 // number of warps on one times a warp's FP64 instructions: `per_case` for each case and
-// about 150 for the geometry. More lanes even out the last round, fewer compute the
+// about 115 for the geometry. More lanes even out the last round, fewer compute the
 // geometry less often.
 inline int f64_case_split(int64_t n_elem, int R, int per_case, int sms, int64_t* cost_out = nullptr) {
   int best = 1;
   int64_t best_cost = INT64_MAX;
   for (int split = 1; split <= 32 && split < 2 * R; split *= 2) {
     const int64_t warps = (n_elem * split + 31) / 32, units = 4 * (int64_t)sms;
-    const int64_t cost = ((warps + units - 1) / units) * ((int64_t)((R + split - 1) / split) * per_case + 150);
+    const int64_t cost = ((warps + units - 1) / units) * ((int64_t)((R + split - 1) / split) * per_case + 115);
     if (cost < best_cost) {
       best_cost = cost;
       best = split;
