@@ -698,9 +698,10 @@ __global__ void k_outer_update(int64_t N, Cases C, double* __restrict__ rv, cons
 
 // The FP64 passes of an outer iteration for even R: thread = (node, 2 cases), 48 contiguous
 // bytes of an FP64 vector in three 16-byte loads. Same arithmetic per value as k_outer_zq,
-// k_outer_p, k_dot, k_outer_update and k_cast_start. Bound by HBM once the FP64 pipe has
-// only the multiply-adds to do (R = 16, 1.41 M nodes, with the conversions there and 8-byte
-// loads: 0.30, 0.30, 0.38, 0.66 and 0.25 ms; (z, r) then needed z a second time).
+// k_dot, k_outer_update and k_cast_start. Bound by HBM once the FP64 pipe has only the
+// multiply-adds to do. R = 16, 1.41 M nodes: (z, q) 0.30, (z, r) and (p, q) 0.38, update 0.66,
+// start 0.25 ms before; (z, q) and (z, r) 0.25, (p, q) 0.15, update 0.53, start 0.18 ms now.
+// (k_outer_p in this form took 0.34 instead of 0.30 ms and stays with one case per thread.)
 __global__ void __launch_bounds__(256) k_outer_zq2(int64_t N, Cases C, const float* __restrict__ ub,
                                                    const double* __restrict__ q, const double* __restrict__ rv) {
   extern __shared__ double sm[];
@@ -731,28 +732,6 @@ __global__ void __launch_bounds__(256) k_dot_f64_2(int64_t N, Cases C, int field
   for (int k = 0; k < 6; ++k) acc[0][k / 3] += x[k] * y[k];
   VEC_LOOP_END
   reduce_cases_w<1, 2>(acc, C.R / 2, sm, {C.d + field * C.R});
-}
-
-__global__ void __launch_bounds__(256) k_outer_p2(int64_t N, Cases C, const float* __restrict__ ub,
-                                                  double* __restrict__ p) {
-  double be[2];
-  bool act[2];
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    const int r = 2 * (threadIdx.x % (C.R / 2)) + c;
-    act[c] = C.I(I_ACTIVE, r);
-    be[c] = C.D(D_BETA, r);
-  }
-  if (!act[0] && !act[1]) return;
-  GROUP_LOOP_BEGIN(2)
-  double z[6], v[6];
-  load6(ub + o, z);
-  load6(p + o, v);
-#pragma unroll
-  for (int k = 0; k < 6; ++k)
-    if (act[k / 3]) v[k] = be[k / 3] != 0.0 ? z[k] + be[k / 3] * v[k] : z[k];
-  store6(p + o, v);
-  VEC_LOOP_END
 }
 
 __global__ void __launch_bounds__(256) k_outer_update2(int64_t N, Cases C, double* __restrict__ rv,
@@ -1511,7 +1490,7 @@ struct Solve {
   // a kernel with two cases per thread (R even) reducing `nf` fields
   template <typename K, typename... A>
   void vec_w(K kern, int nf, A... args) {
-    const VGeom g2 = vgeom_w(N, R, 2, sms, nf > 0 ? 3 : 8);
+    const VGeom g2 = vgeom_w(N, R, 2, sms, 3);
     kern<<<g2.grid, g2.tpb, 2 * (size_t)nf * g2.tpb * sizeof(double), s>>>(N, C, args...);
     FE_CHECK_LAUNCH();
   }
@@ -1621,7 +1600,7 @@ static void level_apply(Solve& S, const Level& L, const float* x, float* y, cons
 // one inner step (Algorithm 1(b)) and the stop test for the next one
 static void inner_step(Solve& S, const Level& L, cudaGraphConditionalHandle loop, int use_loop) {
   if (S.R % 4 == 0) {
-    const VGeom g4 = vgeom_w(L.N, S.R, 4, S.sms), gp = vgeom_w(L.N, S.R, 4, S.sms, 6);
+    const VGeom g4 = vgeom_w(L.N, S.R, 4, S.sms), gp = vgeom_w(L.N, S.R, 4, S.sms, 3);
     const size_t col = 4 * (size_t)g4.tpb * sizeof(double);
     k_inner_p4<<<gp.grid, gp.tpb, 0, S.s>>>(L.N, S.C, L.B, L.eb, L.pb);
     FE_CHECK_LAUNCH();
@@ -1821,8 +1800,7 @@ static void fcg_iteration(Solve& S) {
   if (even) S.vec_w(k_outer_zq2, 2, ub, q, rc);
   else S.vec(k_outer_zq, ub, q, rc);
   S.scal(s_outer_beta, S.o.literal_beta);
-  if (even) S.vec_w(k_outer_p2, 0, ub, w->p.as<double>());
-  else S.vec(k_outer_p, ub, w->p.as<double>());
+  S.vec(k_outer_p, ub, w->p.as<double>());
   ebe_apply<double>(m, S.R, pc, w->q.as<double>(), S.s);
   if (even) S.vec_w(k_dot_f64_2, 1, (int)D_GAM, pc, q);
   else S.vec(k_dot<double>, (int)D_GAM, (const int*)nullptr, pc, q);
