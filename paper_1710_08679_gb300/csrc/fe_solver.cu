@@ -116,8 +116,8 @@ static VGeom vgeom(int64_t N, int R, int sms) {
 
 // the same for kernels with W cases per thread (R a multiple of W): blocks of K*G threads,
 // G = R/W, thread (j, g) handles node block*K + j and cases W g .. W g + W - 1 with 16-byte
-// loads. Reducing kernels: two blocks per SM, enough loads in flight, and fewer blocks do
-// less of the FP64 reduction at the end (an FP64 instruction takes as long as 61 others).
+// loads. Two or three blocks per SM: enough loads in flight, and fewer blocks do less of the
+// FP64 reduction at the end (an FP64 instruction takes as long as 61 others).
 static VGeom vgeom_w(int64_t N, int R, int W, int sms, int per_sm = 2) {
   VGeom g;
   g.R = R;
@@ -528,8 +528,8 @@ __global__ void k_inner_update(int64_t N, Cases C, const float* __restrict__ Bi,
 // The three passes of an inner step for R a multiple of 4: thread = (node, 4 cases), 48
 // contiguous bytes of each vector in three 16-byte loads and the node's block loaded once
 // for four cases. Same arithmetic per value as k_dot, k_inner_p and k_inner_update. Bound
-// by HBM at level 0 (R = 16, 1.41 M nodes: p, dot and update 0.56 -> 0.50 ms) and by L2 at
-// level 1 (0.086 -> 0.073 ms).
+// by HBM at level 0 (R = 16, 1.41 M nodes: p, dot and update 0.56 -> 0.47 ms) and by L2 at
+// level 1 (0.086 -> 0.071 ms).
 #define GROUP_LOOP_BEGIN(W)                               \
   const int R = C.R;                                      \
   const int G = R / W;                                    \
@@ -701,7 +701,8 @@ __global__ void k_outer_update(int64_t N, Cases C, double* __restrict__ rv, cons
 // k_dot, k_outer_update and k_cast_start. Bound by HBM once the FP64 pipe has only the
 // multiply-adds to do. R = 16, 1.41 M nodes: (z, q) 0.30, (z, r) and (p, q) 0.38, update 0.66,
 // start 0.25 ms before; (z, q) and (z, r) 0.25, (p, q) 0.15, update 0.53, start 0.18 ms now.
-// (k_outer_p in this form took 0.34 instead of 0.30 ms and stays with one case per thread.)
+// (k_outer_p
+// in this form took 0.34 instead of 0.24 ms and stays with one case per thread.)
 __global__ void __launch_bounds__(256) k_outer_zq2(int64_t N, Cases C, const float* __restrict__ ub,
                                                    const double* __restrict__ q, const double* __restrict__ rv) {
   extern __shared__ double sm[];
