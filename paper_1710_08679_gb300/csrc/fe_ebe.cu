@@ -137,6 +137,62 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) ebe_direct_kern
   }
 }
 
+// FP32 direct kernel for even R: thread = (element, two cases), the element product in paired
+// FP32 instructions and a node's six values in three 8-byte loads and atomic adds (rows of
+// 3R floats are 8-byte aligned), so the geometry, the arithmetic and the atomics of two
+// cases take the instructions of one. Bound by the atomics: 41x33x18 crust block, R = 6 / 10 /
+// 18 / 30: 86 / 126 / 226 / 368 us with one case per thread, 75 / 112 / 201 / 324 us here.
+__global__ void __launch_bounds__(128, 3) ebe_direct_x2_kernel(MeshView<float> M, int R,
+                                                               const uint16_t* __restrict__ own,
+                                                               const float* __restrict__ x, float* __restrict__ y,
+                                                               const int* __restrict__ skip) {
+  const int P = R / 2;
+  const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if ((skip && *skip) || gid >= M.n_elem * P) return wait_for_zero();
+  const int64_t e = gid / P;
+  const int r = 2 * (int)(gid - e * P);
+  int nd[10];
+  load_conn<float>(M.conn, e, nd);
+  ElemGeo<float> G;
+  load_geometry(M, e, nd, G);
+  float2 u[10][3];
+  unsigned mk = 0;
+#pragma unroll
+  for (int a = 0; a < 10; ++a) {
+    mk |= ((unsigned)__ldg(M.nmask + nd[a]) & 7u) << (3 * a);
+    const float2* q = reinterpret_cast<const float2*>(x + ((int64_t)nd[a] * R + r) * 3);
+    const float2 v0 = __ldg(q), v1 = __ldg(q + 1), v2 = __ldg(q + 2);
+    const float2 w[3] = {make_float2(v0.x, v1.y), make_float2(v0.y, v2.x), make_float2(v1.x, v2.y)};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) u[a][c] = ((mk >> (3 * a + c)) & 1) ? w[c] : make_float2(0.f, 0.f);
+  }
+  float2 yl[10][3];
+  elem_apply_x2(G, u, yl);
+  const int ow = __ldg(own + e);
+  wait_for_zero();
+#pragma unroll
+  for (int a = 0; a < 10; ++a) {
+    const int64_t o = ((int64_t)nd[a] * R + r) * 3;
+    if (((mk >> (3 * a)) & 7u) == 7u) {
+      float2* q = reinterpret_cast<float2*>(y + o);
+      atomicAdd(q, make_float2(yl[a][0].x, yl[a][1].x));
+      atomicAdd(q + 1, make_float2(yl[a][2].x, yl[a][0].y));
+      atomicAdd(q + 2, make_float2(yl[a][1].y, yl[a][2].y));
+    } else {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        if ((mk >> (3 * a + c)) & 1) {
+          atomicAdd(y + o + c, yl[a][c].x);
+          atomicAdd(y + o + 3 + c, yl[a][c].y);
+        } else if ((ow >> a) & 1) {   // constrained DOF: (I - P) x, written once by the node's owner element
+          y[o + c] = __ldg(x + o + c);
+          y[o + 3 + c] = __ldg(x + o + 3 + c);
+        }
+      }
+    }
+  }
+}
+
 // FP64 direct kernel: thread = (element, share of the cases); lane `part` of an
 // element's `split` lanes takes cases part, part + split, ... Bound by the FP64 pipe (1/61
 // of FP32), so the geometry, a fifth of a case's FP64 instructions, is computed once
@@ -1394,11 +1450,15 @@ static void launch_direct(const fe_mesh* m, int R, const T* x, T* y, cudaStream_
     launch_behind_zero(ebe_direct_f64_kernel, blocks, 32, 0, s, M, R, split, m->own_elem.as<uint16_t>(), x, y, skip);
   } else {
     // smaller blocks where the largest would leave SMs with less than four of them
-    const int64_t total = M.n_elem * R;
-    int tpb = kThreads;
+    const bool x2 = R % 2 == 0;
+    const int64_t total = M.n_elem * (x2 ? R / 2 : R);
+    int tpb = x2 ? 128 : kThreads;
     while (tpb > 32 && total < (int64_t)tpb * sms * 4) tpb /= 2;
     const int64_t blocks = (total + tpb - 1) / tpb;
-    launch_behind_zero(ebe_direct_kernel<T>, blocks, tpb, 0, s, M, R, m->own_elem.as<uint16_t>(), x, y, skip);
+    if (x2)
+      launch_behind_zero(ebe_direct_x2_kernel, blocks, tpb, 0, s, M, R, m->own_elem.as<uint16_t>(), x, y, skip);
+    else
+      launch_behind_zero(ebe_direct_kernel<T>, blocks, tpb, 0, s, M, R, m->own_elem.as<uint16_t>(), x, y, skip);
   }
 }
 

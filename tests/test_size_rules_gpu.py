@@ -56,6 +56,22 @@ def test_direct_fp64_product(case, R):
         assert np.array_equal(y[:, r][fixed], x[:, r][fixed])
 
 
+# even R: two cases per thread
+@pytest.mark.gpu
+@pytest.mark.parametrize("R", [1, 2, 5, 6, 14, 30])
+def test_direct_fp32_product(case, R):
+    m, K, M = case
+    x = mg.random_vectors(m.n_nodes, R, seed=50 + R).astype(np.float32).astype(np.float64)
+    M.set_variant(R, "f32", DIRECT, 48)
+    y = M.ebe(cuda(x, torch.float32)).double().cpu().numpy()
+    ref = oracle.spmv(K, x)
+    for r in range(R):
+        assert rel_l2(y[:, r], ref[:, r]) <= TOL32, r
+    fixed = m.free == 0
+    for r in range(R):
+        assert np.array_equal(y[:, r][fixed], x[:, r][fixed])
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("R", [1, 2, 5, 16, 33])
 def test_sensitivities(case, R):
