@@ -1,7 +1,8 @@
 // EBE product y = K_bc x for R cases (Eq. 3, multiple vectors of Sec. 3.1).
 //
 // Several kernels compute the same thing; fe_ebe_tune times them per (R, precision):
-//  * EBE_DIRECT: one thread per (element, case). The thread recomputes the
+//  * EBE_DIRECT: one thread per (element, case) (FP32, even R: two cases; FP64: a share of
+//    the element's cases, or a corner of one on small meshes). The thread recomputes the
 //    element geometry, gathers its 30 inputs straight from global memory (the R
 //    threads of one element read the node's 3R contiguous values together) and
 //    scatters 30 results with atomic adds, as the paper's GPU port does
