@@ -130,7 +130,7 @@ void adjoint_grad(const fe_mesh* m, int R, const double* u, const double* lam, d
   const MeshView<double> M = m->view<double>();
   int sms = 0;
   FE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
-  const int split = f64_case_split(M.n_elem, R, 451, sms);
+  const int split = f64_case_split(M.n_elem, R, 451, sms, false);
   const int64_t blocks = (M.n_elem * split + 31) / 32;
   adjoint_kernel<<<(unsigned)blocks, 32, 0, s>>>(M, R, split, m->perm.as<int64_t>(), u, lam, g);
   FE_CHECK_LAUNCH();

@@ -1440,10 +1440,10 @@ static void launch_direct(const fe_mesh* m, int R, const T* x, T* y, cudaStream_
   int sms = 0;
   FE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
   if constexpr (sizeof(T) == 8) {
-    int64_t cost = 0;
-    const int split = f64_case_split(M.n_elem, R, 438, sms, &cost);
-    const int64_t lanes = 4 * M.n_elem * R, units = 4 * (int64_t)sms;
-    if (((lanes + 31) / 32 + units - 1) / units * 185 < cost) {
+    double cost = 0.0;
+    const int split = f64_case_split(M.n_elem, R, 438, sms, true, &cost);
+    const int64_t lanes = 4 * M.n_elem * R;
+    if (f64_cost((lanes + 31) / 32, 185, sms, true) < cost) {
       launch_behind_zero(ebe_corner_f64_kernel, (lanes + 63) / 64, 64, 0, s, M, R, m->own_elem.as<uint16_t>(), x, y, skip);
       return;
     }
