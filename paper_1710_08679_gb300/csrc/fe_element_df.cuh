@@ -30,21 +30,29 @@ namespace fe {
 // dependencies. With v_mj = 4 u_mj - u_j and u_mm = u_m (so that v_mm = 3 u_m), every
 // corner has the same formula.
 //
-// A multiply-add term of a compensated sum takes 11 operations instead of 12: of the
-// rounded product p added to s, bb = s' - s reached the new sum s'; the rest of the exact
-// product, a b - bb, is one FMA (TwoProd and the second half of TwoSum at once), and
-// s - (s' - bb) and the cross terms complete the error. (Adding the product by an FMA,
-// s' = fl(s + a b), would save one more but count part of it twice where s' cancels.)
-// Subtractions are FMAs with a factor of -1: paired instructions have no negated operands.
-// `pnorm` renormalises where a value becomes an operand or a sum goes on; the order of the
-// error terms and these places keep the error of the product at that of the scalar form
-// (3.11e-15 against 64-bit torch on random vectors; one operation less per term and half
-// as many renormalisations gave 3.26e-15 and 632 instead of 654 us).
+// A multiply-add term of a compensated sum (pacc_add) takes 10 operations instead of 12: of
+// the rounded product p added to s, bb = s' - s reached the new sum s'; the rest of the exact
+// product, a b - bb, is one FMA (TwoProd and the second half of TwoSum at once),
+// s - (s' - bb) completes the error, and the cross terms are added to it. (Adding the product by
+// an FMA, s' = fl(s + a b), would save one more but count part of it twice where s' cancels.)
+// That FMA rounds a remainder as large as the sum's own error. Where the sums cancel, which is
+// in the gradients sum_j v_mj g_j of displacements that are mostly translation, as a solve's
+// are, pacc_add_exact forms both errors without rounding (12 operations), and v_mm = 3 u_m gets
+// the one rounding of a product (p4add). Subtractions are FMAs with a factor of -1: paired
+// instructions have no negated operands. `pnorm` renormalises where a value becomes an
+// operand or a sum goes on.
+//
+// Mean error of an element product against long double, relative to the scalar form's
+// (TwoProd and TwoSum apart, 12 operations a term): random vectors -0.6 %, linear fields
+// -2.8 %, translation and a linear field 0.0 %, slip solutions -0.4 %; whole products on
+// random vectors 3.1e-15 against 64-bit torch. With pacc_add in the gradients too and 3 u_m
+// as 4 u_m - u_m the product takes 1 % less time, and the error of translated fields grows
+// by 8 %.
 //
 // Bound by the FP32 pipe, on which a paired instruction takes two cycles, and by the
-// latencies that four warps per scheduler leave uncovered (ncu: FMA pipe 50 %, issue 50 %;
-// the scalar form issued twice as many instructions at 65 %). R = 16 on the 41x33x18 crust
-// block: 752 -> 656 us, R = 4: 286 -> 234 us; R = 16 on the 70x70x35 block: 5.25 -> 4.45 ms.
+// latencies that four warps per scheduler leave uncovered (ncu: FMA pipe 53 %, issue 50 %;
+// the scalar form issued half as many instructions again at 65 %). R = 16 on the 41x33x18
+// crust block: 750 -> 657 us, R = 4: 283 -> 227 us; R = 16 on the 70x70x35 block: 5.25 -> 4.50 ms.
 //
 // The element's data: for i = 0, 1, 2 the float4 (g0_i.hi, g1_i.hi, g0_i.lo, g1_i.lo) and
 // the same of g2, g3, then (lam'.hi, lam'.lo, mu'.hi, mu'.lo) and (0, 0, 2^e, 0): V/5 =
@@ -94,7 +102,19 @@ FE_HD void pacc_add(dfp& A, const dfp& a, const dfp& b, float2 z) {
   const float2 r = q_sub(A.s, q_add(s, nbb));
   const float2 e = q_add(r, q_fma(a.s, b.s, nbb));     // fl(A.s + p) missed this much of A.s + a b
   A.s = s;
-  A.c = q_add(A.c, q_add(e, q_fma(a.s, b.c, q_mul(a.c, b.s))));
+  A.c = q_add(A.c, q_fma(a.s, b.c, q_fma(a.c, b.s, e)));
+}
+
+// A += a b for sums that cancel (v_mj g_j of a displacement that is nearly a translation),
+// nb = -b.s: the product's and the sum's rounding errors each formed exactly
+FE_HD void pacc_add_exact(dfp& A, const dfp& a, const dfp& b, float2 nb, float2 z) {
+  const float2 np = q_fma(a.s, nb, z);                 // -p
+  const float2 s = q_sub(A.s, np);
+  const float2 nbb = q_sub(A.s, s);
+  const float2 r = q_sub(A.s, q_add(s, nbb));
+  const float2 e = q_add(r, q_sub(nbb, np));           // A.s + p - s
+  A.c = q_add(A.c, q_add(e, q_fma(a.s, b.c, q_fma(a.c, b.s, q_fma(a.s, b.s, np)))));
+  A.s = s;
 }
 
 FE_HD dfp padd(const dfp& a, const dfp& b) {
@@ -104,13 +124,17 @@ FE_HD dfp padd(const dfp& a, const dfp& b) {
   return {s, q_add(e, q_add(a.c, b.c))};
 }
 
-// 4 a - b
-FE_HD dfp p4sub(const dfp& a, const dfp& b) {
-  const float2 a4 = q_mul(a.s, q_bc(4.f));
-  const float2 s = q_sub(a4, b.s);
-  const float2 nbb = q_sub(a4, s);
-  const float2 e = q_add(q_sub(a4, q_add(s, nbb)), q_sub(nbb, b.s));
-  return {s, q_fma(a.c, q_bc(4.f), q_sub(e, b.c))};
+// 4 a + b. In lane M (0: x, 1: y, -1: none) b = -a: there the low part 3 a.c + e (e: what
+// the sum of the high parts missed) has one rounding, as the product 3 a has.
+template <int M>
+FE_HD dfp p4add(const dfp& a, const dfp& b) {
+  const float2 s = q_fma(a.s, q_bc(4.f), b.s);
+  const float2 bb = q_fma(a.s, q_bc(-4.f), s);
+  const float2 r = q_fma(a.s, q_bc(4.f), q_sub(bb, s));
+  const float2 e = q_add(r, q_sub(b.s, bb));
+  const float2 k = make_float2(M == 0 ? 3.f : 4.f, M == 1 ? 3.f : 4.f);
+  const float2 t = q_fma(a.c, k, make_float2(M == 0 ? e.x : b.c.x, M == 1 ? e.y : b.c.y));
+  return {s, q_add(t, make_float2(M == 0 ? 0.f : e.x, M == 1 ? 0.f : e.y))};
 }
 
 FE_HD dfp pscale(const dfp& a, float k) { return {q_mul(a.s, q_bc(k)), q_mul(a.c, q_bc(k))}; }
@@ -125,21 +149,23 @@ FE_HD dfp geo_both(const float4* gs, int i) {
 template <int P, int J>
 FE_HD void pair_gradient_term(const float4* gs, const df* xa, const int* off, float2 z, dfp A[3][3]) {
   constexpr int e0 = edge_or_corner(2 * P, J), e1 = edge_or_corner(2 * P + 1, J);
+  constexpr int own = J == 2 * P ? 0 : J == 2 * P + 1 ? 1 : -1;   // the lane with 3 u_m
   dfp v[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const df uj = xa[off[J] + a];
-    v[a] = pnorm(p4sub(p_pack(xa[off[e0] + a], xa[off[e1] + a]), p_pack(uj, uj)));
+    v[a] = pnorm(p4add<own>(p_pack(xa[off[e0] + a], xa[off[e1] + a]), {q_bc(-uj.hi), q_bc(-uj.lo)}));
   }
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
     const dfp g = geo_both<J>(gs, b);
+    const float2 ng = q_bc(-g.s.x);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       if (J == 0)
         pacc_first(A[a][b], v[a], g, z);
       else
-        pacc_add(A[a][b], v[a], g, z);
+        pacc_add_exact(A[a][b], v[a], g, ng, z);
     }
   }
 }
