@@ -298,7 +298,8 @@ fe_status fe_ebe_tune(fe_mesh* mesh, int32_t R, fe_dtype dtype, void* stream, in
  * fe_pcg_solve -- solve K_bc u_r = f_r for R cases at once (Algorithm 1 with the
  * inner loop at level 0 only, or plain block-Jacobi PCG).
  *   f_dev    device double [N][R][3]; constrained entries are ignored (treated as 0)
- *   u_dev    device double [N][R][3]; in: initial guess, out: solution
+ *   u_dev    device double [N][R][3]; in: initial guess, out: solution. An 8-byte
+ *            aligned u_dev is accepted too (some passes over it are slower)
  *   opts     host; NULL = defaults
  *   stats    host [R], written on return
  * Synchronous: returns when u and stats are final. Each case stops on its own

@@ -1481,6 +1481,7 @@ struct Solve {
   cudaStream_t s;
   const double* f;
   double* u;
+  bool u_aligned = true;   // to 16 bytes, as the products' vector loads need it
   fe_solve_opts o;
 
   template <typename K, typename... A>
@@ -1806,7 +1807,7 @@ static void fcg_iteration(Solve& S) {
   if (even) S.vec_w(k_dot_f64_2, 1, (int)D_GAM, pc, q);
   else S.vec(k_dot<double>, (int)D_GAM, (const int*)nullptr, pc, q);
   S.scal(s_outer_alpha);
-  if (even && ((uintptr_t)S.u & 15) == 0)   // the caller's u has no alignment rule
+  if (even && S.u_aligned)
     S.vec_w(k_outer_update2, 1, w->r.as<double>(), q, S.u, pc);
   else
     S.vec(k_outer_update, w->r.as<double>(), q, S.u, pc);
@@ -1878,6 +1879,7 @@ static fe_status run_solve(fe_mesh* m, int R, const double* f, double* u, const 
   S.s = s;
   S.f = f;
   S.u = u;
+  S.u_aligned = ((uintptr_t)u & 15) == 0;
   S.o = o;
   const bool pcg = o.solver == FE_SOLVER_PCG64;
   if (o.solver == FE_SOLVER_FCG_MG || o.solver == FE_SOLVER_FCG_AMG) {
@@ -1923,7 +1925,12 @@ static fe_status run_solve(fe_mesh* m, int R, const double* f, double* u, const 
   // start: u = P u, r = P f - K u, ||f||, ||r|| (the product is skipped when u = 0)
   S.scal(s_init);
   S.vec(k_prepare, m->nmask.as<uint8_t>(), f, u);
-  ebe_apply<double>(m, R, u, w->q.as<double>(), s, S.C.done + 2);
+  const double* x0 = u;
+  if (!S.u_aligned) {
+    x0 = w->p.as<double>();
+    FE_CUDA(cudaMemcpyAsync(w->p.ptr, u, (size_t)S.N * R * 3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
+  }
+  ebe_apply<double>(m, R, x0, w->q.as<double>(), s, S.C.done + 2);
   S.vec(k_residual, m->nmask.as<uint8_t>(), f, (const double*)w->q.as<double>(), w->r.as<double>());
   S.scal(s_start, o.tol, 0);
   S.vec(k_zero_trivial, u);
@@ -1962,11 +1969,12 @@ static fe_status run_solve(fe_mesh* m, int R, const double* f, double* u, const 
       FE_CUDA(cudaMemcpyAsync(hd.data(), w->d.ptr, hd.size() * 8, cudaMemcpyDeviceToHost, s));
       FE_CUDA(cudaStreamSynchronize(s));
       // confirm candidates with the true FP64 residual: one all-case product when
-      // a quarter or more of the cases are candidates, else one product per case
+      // a quarter or more of the cases are candidates (and u can be its input), else
+      // one product per case
       bool any_active = false, restart = false;
       int n_cand = 0;
       for (int c = 0; c < R; ++c) n_cand += hi[I_CAND * R + c] ? 1 : 0;
-      const bool batched = R > 1 && 4 * n_cand >= R;
+      const bool batched = R > 1 && 4 * n_cand >= R && S.u_aligned;
       if (batched) {
         if (!w->tall.ptr) w->tall.alloc((size_t)S.N * R * 3 * sizeof(double));
         ebe_apply<double>(m, R, u, w->tall.as<double>(), s);
