@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "fe.h"
+#include "fe_rules.cuh"
 
 namespace fe {
 

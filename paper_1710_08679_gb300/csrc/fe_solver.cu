@@ -117,13 +117,15 @@ static VGeom vgeom(int64_t N, int R, int sms) {
 // the same for kernels with W cases per thread (R a multiple of W): blocks of K*G threads,
 // G = R/W, thread (j, g) handles node block*K + j and cases W g .. W g + W - 1 with 16-byte
 // loads. Two or three blocks per SM: enough loads in flight, and fewer blocks do less of the
-// FP64 reduction at the end (an FP64 instruction takes as long as 61 others).
+// FP64 reduction at the end (an FP64 instruction takes as long as 61 others). Smaller blocks
+// on small meshes, as above: step of the inner loop on 24,389 nodes, R = 4, 32.3 -> 31.0 us.
 static VGeom vgeom_w(int64_t N, int R, int W, int sms, int per_sm = 2) {
   VGeom g;
   g.R = R;
   g.K = 1;
   const int G = R / W;
   while (g.K * 2 * G <= 256) g.K *= 2;
+  while (g.K > 1 && g.K * G > 32 && (N + g.K - 1) / g.K < sms) g.K /= 2;
   g.tpb = g.K * G;
   const int64_t need = (N + g.K - 1) / g.K;
   const int64_t cap = (int64_t)sms * per_sm;
@@ -525,11 +527,11 @@ __global__ void k_inner_update(int64_t N, Cases C, const float* __restrict__ Bi,
   reduce_cases((double)a2, C.R, blockDim.x / C.R, sm, C.d + D_RHOA * C.R);
 }
 
-// The three passes of an inner step for R a multiple of 4: thread = (node, 4 cases), 48
-// contiguous bytes of each vector in three 16-byte loads and the node's block loaded once
-// for four cases. Same arithmetic per value as k_dot, k_inner_p and k_inner_update. Bound
-// by HBM at level 0 (R = 16, 1.41 M nodes: p, dot and update 0.56 -> 0.47 ms) and by L2 at
-// level 1 (0.086 -> 0.071 ms).
+// The three passes of an inner step with four cases per thread (four_case_passes): thread =
+// (node, 4 cases), 48 contiguous bytes of each vector in three 16-byte loads and the node's
+// block loaded once for four cases. Same arithmetic per value as k_dot, k_inner_p and
+// k_inner_update. Bound by HBM at level 0 (R = 16, 1.41 M nodes: p, dot and update 0.56 ->
+// 0.47 ms) and by L2 at level 1 (0.086 -> 0.071 ms).
 #define GROUP_LOOP_BEGIN(W)                               \
   const int R = C.R;                                      \
   const int G = R / W;                                    \
@@ -1601,7 +1603,7 @@ static void level_apply(Solve& S, const Level& L, const float* x, float* y, cons
 
 // one inner step (Algorithm 1(b)) and the stop test for the next one
 static void inner_step(Solve& S, const Level& L, cudaGraphConditionalHandle loop, int use_loop) {
-  if (S.R % 4 == 0) {
+  if (four_case_passes(L.N, S.R, S.sms)) {
     const VGeom g4 = vgeom_w(L.N, S.R, 4, S.sms), gp = vgeom_w(L.N, S.R, 4, S.sms, 3);
     const size_t col = 4 * (size_t)g4.tpb * sizeof(double);
     k_inner_p4<<<gp.grid, gp.tpb, 0, S.s>>>(L.N, S.C, L.B, L.eb, L.pb);
