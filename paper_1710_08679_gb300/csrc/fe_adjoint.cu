@@ -14,11 +14,11 @@ namespace fe {
 
 namespace {
 
-constexpr int kThreads = 128;
-
 // Corner strains of one field, e[m] = (xx, yy, zz, 2 yz, 2 xz, 2 xy) of grad u at corner
 // m: v_mm = 3 u_m (the factor in g3 = 3 g) and v_mj = 4 u_mj - u_j as in elem_apply, summed
-// straight into the symmetric components.
+// straight into the symmetric components. The multiply-adds are written out: left to itself
+// the compiler forms 4 u_mj once for both ends of an edge and subtracts, 108 instructions a case
+// for 72 (522 in all; the product, whose 4 u_mj it does fold, has 440).
 __device__ __forceinline__ void corner_strain(const double g[4][3], const double g3[4][3], const double u[10][3], int m,
                                               double e[6]) {
 #pragma unroll
@@ -28,7 +28,7 @@ __device__ __forceinline__ void corner_strain(const double g[4][3], const double
     double v[3];
     const double* w = j == m ? g3[j] : g[j];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) v[a] = j == m ? u[m][a] : 4.0 * u[edge_or_corner(m, j)][a] - u[j][a];
+    for (int a = 0; a < 3; ++a) v[a] = j == m ? u[m][a] : fma(4.0, u[edge_or_corner(m, j)][a], -u[j][a]);
 #pragma unroll
     for (int a = 0; a < 3; ++a) e[a] = fma(v[a], w[a], e[a]);
     e[3] = fma(v[1], w[2], fma(v[2], w[1], e[3]));
@@ -50,10 +50,11 @@ __device__ __forceinline__ void strain_energy(const double e[6], const double f[
 // Bound by the FP64 pipe (1/61 of FP32), so what counts is the number of FP64
 // instructions. lambda_e^T K_e u_e is evaluated as the strain energy
 //   V/20 [ sum_m s_m : e'_m + (sum_m s_m) : (sum_m e'_m) ],  s = lam tr(e) I + 2 mu e,
-// with lam and mu applied after the sum over the cases: about 450 instructions per case,
-// where forming K_e u_e and its product with lambda_e took about 490. One-warp blocks and
+// with lam and mu applied after the sum over the cases: 475 instructions per case (ncu),
+// where forming K_e u_e and its product with lambda_e takes 511. One-warp blocks and
 // the split (f64_case_split) even out the last round. 16 cases on the 82,944 elements of the
-// 24^3 box: 1418 -> 1296 us; error against 64-bit torch 4.06e-16 (before 4.36e-16).
+// 24^3 box: 1418 us in that form, 1171 us here (1296 us with 522 instructions per case);
+// 1,029,000 elements: 14.88 and 13.62 ms. Error against 64-bit torch 4.06e-16 (4.36e-16).
 __global__ void __launch_bounds__(32) adjoint_kernel(MeshView<double> M, int R, int split,
                                                      const int64_t* __restrict__ perm, const double* __restrict__ u,
                                                      const double* __restrict__ lam, double* __restrict__ g) {
