@@ -52,7 +52,7 @@ __device__ __forceinline__ void strain_energy(const double e[6], const double f[
 //   V/20 [ sum_m s_m : e'_m + (sum_m s_m) : (sum_m e'_m) ],  s = lam tr(e) I + 2 mu e,
 // with lam and mu applied after the sum over the cases: 475 instructions per case (ncu),
 // where forming K_e u_e and its product with lambda_e takes 511. One-warp blocks and
-// the split (f64_case_split) even out the last round. 16 cases on the 82,944 elements of the
+// the split (f64_adjoint_split) even out the last round. 16 cases on the 82,944 elements of the
 // 24^3 box: 1418 us in that form, 1171 us here (1296 us with 522 instructions per case);
 // 1,029,000 elements: 14.88 and 13.62 ms. Error against 64-bit torch 4.06e-16 (4.36e-16).
 __global__ void __launch_bounds__(32) adjoint_kernel(MeshView<double> M, int R, int split,
@@ -131,7 +131,7 @@ void adjoint_grad(const fe_mesh* m, int R, const double* u, const double* lam, d
   const MeshView<double> M = m->view<double>();
   int sms = 0;
   FE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
-  const int split = f64_case_split(M.n_elem, R, 451, sms, false);
+  const int split = f64_adjoint_split(M.n_elem, R, sms);
   const int64_t blocks = (M.n_elem * split + 31) / 32;
   adjoint_kernel<<<(unsigned)blocks, 32, 0, s>>>(M, R, split, m->perm.as<int64_t>(), u, lam, g);
   FE_CHECK_LAUNCH();

@@ -195,9 +195,9 @@ __global__ void __launch_bounds__(128, 3) ebe_direct_x2_kernel(MeshView<float> M
 }
 
 // FP64 direct kernel: thread = (element, share of the cases); lane `part` of an
-// element's `split` lanes takes cases part, part + split, ... Bound by the FP64 pipe (1/61
-// of FP32), so the geometry, a fifth of a case's FP64 instructions, is computed once
-// per thread, and blocks of one warp fill the SMs evenly. 5 cases on the 146,124 elements of
+// element's `split` lanes (f64_direct_split) takes cases part, part + split, ... Bound by the
+// FP64 pipe (1/61 of FP32), so the geometry, a fifth of a case's FP64 instructions, is computed
+// once per thread, and blocks of one warp fill the SMs evenly. 5 cases on the 146,124 elements of
 // the 41x33x18 crust block: 812 -> 678 us; one case on the 1.03 M elements of the 70x70x35
 // block: 1142 -> 980 us (0.92 TFLOP/s of 1.2), 50 us of it from the stored Lame constants.
 __global__ void __launch_bounds__(32) ebe_direct_f64_kernel(MeshView<double> M, int R, int split,
@@ -1440,10 +1440,9 @@ static void launch_direct(const fe_mesh* m, int R, const T* x, T* y, cudaStream_
   int sms = 0;
   FE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
   if constexpr (sizeof(T) == 8) {
-    double cost = 0.0;
-    const int split = f64_case_split(M.n_elem, R, 438, sms, true, &cost);
-    const int64_t lanes = 4 * M.n_elem * R;
-    if (f64_cost((lanes + 31) / 32, 185, sms, true) < cost) {
+    const int split = f64_direct_split(M.n_elem, R, sms);
+    if (split == 0) {
+      const int64_t lanes = 4 * M.n_elem * R;
       launch_behind_zero(ebe_corner_f64_kernel, (lanes + 63) / 64, 64, 0, s, M, R, m->own_elem.as<uint16_t>(), x, y, skip);
       return;
     }

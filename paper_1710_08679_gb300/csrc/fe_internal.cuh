@@ -312,35 +312,6 @@ void grid_wait_selftest(const fe_mesh* m, long long cycles, cudaStream_t s);  //
 // Block Jacobi (fe_solver.cu)
 void build_block_jacobi(fe_mesh* m, cudaStream_t s);
 
-// Time of `warps` warps of `instr` FP64 instructions each, in instructions: each of the
-// 4 * sms SM sub-partitions runs its warps through its FP64 unit one instruction after the
-// other. The products' warps, which wait on scattered loads and atomics, end about one
-// warp's time after the average (`spread`; 5 cases on 7,986 elements: 60 us by this rule,
-// 89 by the other, 91 before); those of the sensitivities take the fullest sub-partition's
-// time (9 cases on 31,104 elements: 292 us, 365 by the spread rule, 325 before).
-inline double f64_cost(int64_t warps, int instr, int sms, bool spread) {
-  const int64_t units = 4 * (int64_t)sms;
-  return (spread ? (double)warps / (double)units + 1.0 : (double)((warps + units - 1) / units)) * instr;
-}
-
-// Lanes an element's R cases are spread over in the FP64 kernels whose threads loop over
-// cases (a power of two at most 32): `per_case` FP64 instructions for each case and about
-// 115 for the geometry. More lanes fill the sub-partitions evenly, fewer compute the
-// geometry less often.
-inline int f64_case_split(int64_t n_elem, int R, int per_case, int sms, bool spread, double* cost_out = nullptr) {
-  int best = 1;
-  double best_cost = 1e300;
-  for (int split = 1; split <= 32 && split < 2 * R; split *= 2) {
-    const double cost = f64_cost((n_elem * split + 31) / 32, (R + split - 1) / split * per_case + 115, sms, spread);
-    if (cost < best_cost) {
-      best_cost = cost;
-      best = split;
-    }
-  }
-  if (cost_out) *cost_out = best_cost;
-  return best;
-}
-
 // Adjoint (fe_adjoint.cu)
 void adjoint_grad(const fe_mesh* m, int R, const double* u, const double* lam, double* g, cudaStream_t s);
 

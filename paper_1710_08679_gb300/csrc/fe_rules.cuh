@@ -4,7 +4,58 @@
 
 #include <stdint.h>
 
+#include <algorithm>
+#include <cmath>
+
 namespace fe {
+
+// Rounds that `warps` warps of equal length take on the 4 * sms SM sub-partitions, each of
+// which runs its warps through its FP64 unit one instruction after the other: the number on
+// the fullest one. (Fewer warps than sub-partitions do not go one to each: some share one.)
+inline double f64_rounds(int64_t warps, int sms) {
+  const double n = (double)warps / (4.0 * sms);
+  return n > 1.0 ? std::ceil(n) : 1.0 + 0.4 * std::max(0.0, n - 0.3);
+}
+
+// Lanes an element's R cases are spread over in the FP64 kernels whose threads loop over
+// cases: `per_case` FP64 instructions' time for each case and `geometry` for the element. More
+// lanes fill the sub-partitions evenly, fewer compute the geometry less often. `pow2`: the
+// lanes' sums meet by shuffles, so their number is a power of two of at most 32.
+inline int f64_case_split(int64_t n_elem, int R, int per_case, int geometry, int sms, bool pow2,
+                          double* cost_out = nullptr) {
+  int best = 1;
+  double best_cost = 1e300;
+  for (int k = R; k >= 1; --k) {   // cases per lane
+    int split = (R + k - 1) / k;
+    while (pow2 && (split & (split - 1)) != 0) ++split;
+    if (pow2 && split > 32) continue;
+    const double cost = f64_rounds((n_elem * split + 31) / 32, sms) * (k * per_case + geometry);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = split;
+    }
+  }
+  if (cost_out) *cost_out = best_cost;
+  return best;
+}
+
+// FP64 direct product: lanes per element, 0 for the kernel with a lane per corner of every
+// (element, case). The times of a case (480: 440 instructions and the waits on its loads),
+// the geometry (70) and a corner (190) were fitted to 9 meshes of 750 to 146,124 elements, R = 1
+// to 64, every split, launched behind the zero pass and in graphs: the choice takes 0.3 and
+// 0.8 % longer than the fastest split on average. us in a graph with 1 / 2 / 4 / R lanes / corners:
+// 3,072 elements, R = 12: 207 / 110 / 57 / 42 / 53; 16,464, R = 9: 172 / 155 / - / 152 / 192.
+inline int f64_direct_split(int64_t n_elem, int R, int sms) {
+  double cost = 0.0;
+  const int split = f64_case_split(n_elem, R, 480, 70, sms, false, &cost);
+  return f64_rounds((4 * n_elem * R + 31) / 32, sms) * 190 < cost ? 0 : split;
+}
+
+// Sensitivities: lanes per element (475 instructions a case; the choice takes 0.3 % longer
+// than the fastest split on average over the same meshes and R).
+inline int f64_adjoint_split(int64_t n_elem, int R, int sms) {
+  return f64_case_split(n_elem, R, 500, 110, sms, true);
+}
 
 // Inner-loop vector passes with four cases per thread: from 140 such threads per SM on.
 // With fewer the SMs are filled better by a thread per case. Step of the inner loop at level

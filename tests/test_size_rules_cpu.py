@@ -16,6 +16,8 @@ SMS = 152
 HARNESS = r"""
 #include "fe_rules.cuh"
 extern "C" int four_case_passes(long n, int R, int sms) { return fe::four_case_passes(n, R, sms); }
+extern "C" int f64_direct_split(long n, int R, int sms) { return fe::f64_direct_split(n, R, sms); }
+extern "C" int f64_adjoint_split(long n, int R, int sms) { return fe::f64_adjoint_split(n, R, sms); }
 """
 
 
@@ -49,3 +51,43 @@ def test_passes_of_four_cases(rules, n, R, one, four):
 @pytest.mark.parametrize("R", [1, 2, 6, 13])
 def test_passes_of_four_cases_need_a_multiple_of_four(rules, R):
     assert not rules.four_case_passes(ctypes.c_long(10**7), R, SMS)
+
+
+# us per FP64 direct product by lanes per element (0: a lane per corner), the fastest few
+@pytest.mark.parametrize("n_elem,R,times", [
+    (750, 1, {0: 11.1, 1: 22.9}),
+    (750, 48, {48: 41.0, 24: 42.4, 0: 53.3, 16: 56.1, 12: 73.1, 10: 91.8, 8: 107.1}),
+    (3072, 1, {0: 11.5, 1: 23.1}),
+    (3072, 8, {8: 32.7, 4: 40.2, 0: 40.9, 3: 57.9, 2: 75.1, 1: 140.0}),
+    (3072, 12, {12: 41.8, 6: 43.1, 0: 53.4, 4: 56.9, 3: 75.2, 2: 110.3, 1: 207.3}),
+    (3072, 24, {12: 73.4, 24: 79.1, 6: 79.9, 8: 84.7, 5: 97.8, 0: 101.7, 4: 107.7}),
+    (7986, 9, {9: 79.8, 3: 83.6, 0: 96.0, 2: 99.3, 5: 104.1, 1: 164.7}),
+    (7986, 18, {9: 143.8, 18: 151.6, 4: 154.1, 6: 159.3, 3: 160.3, 2: 171.8, 0: 186.5}),
+    (16464, 1, {1: 25.8, 0: 27.0}),
+    (16464, 9, {9: 152.3, 2: 155.1, 3: 159.9, 1: 172.2, 5: 178.3, 0: 192.5}),
+    (31104, 9, {3: 264.6, 1: 277.6, 9: 279.5, 5: 283.9, 2: 338.2, 0: 356.0}),
+    (50544, 5, {5: 245.3, 1: 265.7, 3: 282.9, 2: 309.7, 0: 320.1}),
+    (73728, 16, {2: 1060.7, 8: 1068.0, 1: 1070.6, 4: 1070.7, 16: 1115.2, 6: 1169.3, 3: 1192.4}),
+    (146124, 5, {1: 676.6, 5: 698.1, 2: 795.5, 3: 795.5}),
+    (146124, 30, {5: 3751.6, 3: 3761.9, 6: 3767.5, 10: 3805.3, 2: 3826.1, 15: 3877.0, 1: 3928.4})])
+def test_lanes_of_the_fp64_product(rules, n_elem, R, times):
+    assert near_best(rules.f64_direct_split(ctypes.c_long(n_elem), R, SMS), times)
+
+
+# us per sensitivity pass by lanes per element
+@pytest.mark.parametrize("n_elem,R,times", [
+    (750, 9, {16: 21.7, 8: 37.8, 4: 52.3, 2: 81.2, 1: 142.4}),
+    (3072, 9, {4: 52.2, 8: 58.6, 16: 60.4, 2: 83.0, 1: 142.6}),
+    (3072, 24, {8: 84.9, 4: 97.3, 16: 107.9, 32: 114.0, 2: 188.0, 1: 368.2}),
+    (7986, 5, {2: 56.3, 4: 66.4, 8: 77.1, 1: 82.8}),
+    (7986, 16, {4: 123.6, 16: 132.8, 2: 138.3, 8: 142.4, 1: 249.2}),
+    (16464, 3, {1: 56.2, 2: 66.3, 4: 77.1}),
+    (16464, 16, {2: 238.1, 8: 244.8, 16: 261.0, 4: 269.2, 1: 275.2}),
+    (31104, 9, {1: 267.1, 2: 332.7, 4: 354.9, 8: 448.4, 16: 481.2}),
+    (73728, 2, {1: 140.9, 2: 149.0}),
+    (73728, 30, {1: 1933.2, 2: 1936.1, 8: 2049.7, 4: 2077.6, 16: 2093.6, 32: 2249.7}),
+    (82944, 16, {2: 1173.1, 4: 1177.9, 8: 1198.8, 16: 1265.4, 1: 1298.0}),
+    (146124, 16, {4: 2030.4, 2: 2037.4, 1: 2067.5, 8: 2084.6, 16: 2216.8}),
+    (1029000, 16, {1: 13620.4, 2: 13726.2, 4: 13958.7, 8: 14459.7, 16: 15506.9})])
+def test_lanes_of_the_sensitivities(rules, n_elem, R, times):
+    assert near_best(rules.f64_adjoint_split(ctypes.c_long(n_elem), R, SMS), times)
