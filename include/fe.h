@@ -211,10 +211,10 @@ fe_status fe_ebe_apply(const fe_mesh* mesh, int32_t R, fe_dtype dtype, const voi
 fe_status fe_ebe_apply_host(fe_mesh* mesh, int32_t R, fe_dtype dtype, const void* x_host, void* y_host, void* stream);
 
 /* EBE kernel variants (all compute fe_ebe_apply's result):
- *   FE_EBE_DIRECT  one thread per (element, case) (FP32, even R: two cases; FP64: a
- *                  share of an element's cases, or one of its corners on small
- *                  meshes), inputs gathered from global memory, results added with
- *                  global atomics (the paper's GPU port keeps atomics rather than
+ *   FE_EBE_DIRECT  one thread per (element, case) (FP32, even R on large meshes: two
+ *                  cases; FP64: a share of an element's cases, or one of its corners
+ *                  on small meshes), inputs gathered from global memory, results added
+ *                  with global atomics (the paper's GPU port keeps atomics rather than
  *                  element colouring, Sec. 3.2.2);
  *   FE_EBE_TILED   consecutive elements (in the library's locality order) form a
  *                  tile; the tile's node values are staged in shared memory, the

@@ -1,8 +1,8 @@
 // EBE product y = K_bc x for R cases (Eq. 3, multiple vectors of Sec. 3.1).
 //
 // Several kernels compute the same thing; fe_ebe_tune times them per (R, precision):
-//  * EBE_DIRECT: one thread per (element, case) (FP32, even R: two cases; FP64: a share of
-//    the element's cases, or a corner of one on small meshes). The thread recomputes the
+//  * EBE_DIRECT: one thread per (element, case) (FP32, even R on large meshes: two cases;
+//    FP64: a share of the element's cases, or a corner of one on small meshes). The thread recomputes the
 //    element geometry, gathers its 30 inputs straight from global memory (the R
 //    threads of one element read the node's 3R contiguous values together) and
 //    scatters 30 results with atomic adds, as the paper's GPU port does
@@ -91,43 +91,37 @@ __device__ __forceinline__ void load_geometry(const MeshView<T>& M, int64_t e, c
 }
 
 // ---------------------------------------------------------------------------
-// direct kernel: thread = (element, case)
+// FP32 direct kernel: thread = (element, case), 16 warps per SM (128 registers). One-warp
+// blocks spread the last round of warps over all SMs: 16 cases on 7,986 elements in a graph
+// 14.7 us with 256-thread blocks, 13.5 us here; 73,728 elements 85.1 and 81.9 us.
 // ---------------------------------------------------------------------------
-// FP32 (FP64: ebe_direct_f64_kernel): at most 128 registers so that two 256-thread blocks
-// fit per SM
-template <typename T>
-struct MinBlocks {
-  static constexpr int value = sizeof(T) == 4 ? 2 : 1;
-};
-
-template <typename T>
-__global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) ebe_direct_kernel(MeshView<T> M, int R, const uint16_t* __restrict__ own,
-                                                              const T* __restrict__ x, T* __restrict__ y,
-                                                              const int* __restrict__ skip) {
-  const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(32, 16) ebe_direct_kernel(MeshView<float> M, int R, const uint16_t* __restrict__ own,
+                                                            const float* __restrict__ x, float* __restrict__ y,
+                                                            const int* __restrict__ skip) {
+  const int64_t gid = blockIdx.x * (int64_t)32 + threadIdx.x;
   if ((skip && *skip) || gid >= M.n_elem * R) return wait_for_zero();
   const int64_t e = gid / R;
   const int r = (int)(gid - e * R);
   int nd[10];
-  load_conn<T>(M.conn, e, nd);
-  ElemGeo<T> G;
+  load_conn<float>(M.conn, e, nd);
+  ElemGeo<float> G;
   load_geometry(M, e, nd, G);
-  T u[10][3];
+  float u[10][3];
   int mk[10];
 #pragma unroll
   for (int a = 0; a < 10; ++a) {
     mk[a] = __ldg(M.nmask + nd[a]);
-    const T* xa = x + ((int64_t)nd[a] * R + r) * 3;
+    const float* xa = x + ((int64_t)nd[a] * R + r) * 3;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) u[a][c] = ((mk[a] >> c) & 1) ? __ldg(xa + c) : T(0);
+    for (int c = 0; c < 3; ++c) u[a][c] = ((mk[a] >> c) & 1) ? __ldg(xa + c) : 0.f;
   }
-  T yl[10][3];
+  float yl[10][3];
   elem_apply(G, u, yl);
   const int ow = __ldg(own + e);
   wait_for_zero();
 #pragma unroll
   for (int a = 0; a < 10; ++a) {
-    T* ya = y + ((int64_t)nd[a] * R + r) * 3;
+    float* ya = y + ((int64_t)nd[a] * R + r) * 3;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       if ((mk[a] >> c) & 1)
@@ -138,17 +132,19 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) ebe_direct_kern
   }
 }
 
-// FP32 direct kernel for even R: thread = (element, two cases), the element product in paired
-// FP32 instructions and a node's six values in three 8-byte loads and atomic adds (rows of
-// 3R floats are 8-byte aligned), so the geometry, the arithmetic and the atomics of two
-// cases take the instructions of one. Bound by the atomics: 41x33x18 crust block, R = 6 / 10 /
-// 18 / 30: 86 / 126 / 226 / 368 us with one case per thread, 75 / 112 / 201 / 324 us here.
-__global__ void __launch_bounds__(128, 3) ebe_direct_x2_kernel(MeshView<float> M, int R,
+// FP32 direct kernel for even R (direct_two_cases): thread = (element, two cases), the element
+// product in paired FP32 instructions and a node's six values in three 8-byte loads and atomic
+// adds (rows of 3R floats are 8-byte aligned), so the geometry, the arithmetic and the atomics
+// of two cases take the instructions of one. Bound by the atomics on large meshes; 12 warps per
+// SM take 168 registers a thread, 140 bytes of which spill. 41x33x18 crust block in a graph,
+// R = 6 / 10 / 18 / 30: 78 / 118 / 214 / 347 us with one case per thread, 72 / 108 / 196 /
+// 317 us here.
+__global__ void __launch_bounds__(32, 12) ebe_direct_x2_kernel(MeshView<float> M, int R,
                                                                const uint16_t* __restrict__ own,
                                                                const float* __restrict__ x, float* __restrict__ y,
                                                                const int* __restrict__ skip) {
   const int P = R / 2;
-  const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t gid = blockIdx.x * (int64_t)32 + threadIdx.x;
   if ((skip && *skip) || gid >= M.n_elem * P) return wait_for_zero();
   const int64_t e = gid / P;
   const int r = 2 * (int)(gid - e * P);
@@ -387,6 +383,12 @@ __global__ void __launch_bounds__(64) ebe_corner_f64_kernel(MeshView<double> M, 
 // stream, so each free value of y is read, increased and written by one thread
 // at a time: no atomics, and the summation order is fixed (deterministic y).
 // ---------------------------------------------------------------------------
+// FP32: at most 128 registers so that two 256-thread blocks fit per SM
+template <typename T>
+struct MinBlocks {
+  static constexpr int value = sizeof(T) == 4 ? 2 : 1;
+};
+
 template <typename T>
 __global__ void __launch_bounds__(kThreads, MinBlocks<T>::value) ebe_colour_kernel(
     MeshView<T> M, int R, const int32_t* __restrict__ elems, int64_t n, const uint16_t* __restrict__ own,
@@ -1449,16 +1451,13 @@ static void launch_direct(const fe_mesh* m, int R, const T* x, T* y, cudaStream_
     const int64_t blocks = (M.n_elem * split + 31) / 32;
     launch_behind_zero(ebe_direct_f64_kernel, blocks, 32, 0, s, M, R, split, m->own_elem.as<uint16_t>(), x, y, skip);
   } else {
-    // smaller blocks where the largest would leave SMs with less than four of them
-    const bool x2 = R % 2 == 0;
-    const int64_t total = M.n_elem * (x2 ? R / 2 : R);
-    int tpb = x2 ? 128 : kThreads;
-    while (tpb > 32 && total < (int64_t)tpb * sms * 4) tpb /= 2;
-    const int64_t blocks = (total + tpb - 1) / tpb;
+    // blocks of one warp: the last round of warps is spread over all SMs
+    const bool x2 = direct_two_cases(M.n_elem, R);
+    const int64_t blocks = (M.n_elem * (x2 ? R / 2 : R) + 31) / 32;
     if (x2)
-      launch_behind_zero(ebe_direct_x2_kernel, blocks, tpb, 0, s, M, R, m->own_elem.as<uint16_t>(), x, y, skip);
+      launch_behind_zero(ebe_direct_x2_kernel, blocks, 32, 0, s, M, R, m->own_elem.as<uint16_t>(), x, y, skip);
     else
-      launch_behind_zero(ebe_direct_kernel<T>, blocks, tpb, 0, s, M, R, m->own_elem.as<uint16_t>(), x, y, skip);
+      launch_behind_zero(ebe_direct_kernel, blocks, 32, 0, s, M, R, m->own_elem.as<uint16_t>(), x, y, skip);
   }
 }
 

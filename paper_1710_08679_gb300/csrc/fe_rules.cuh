@@ -9,6 +9,14 @@
 
 namespace fe {
 
+// FP32 direct product: two cases per thread (paired instructions) or one. Two halve the
+// geometry and the arithmetic's instructions, at 168 registers a thread instead of 128: worth it
+// on large meshes; on small ones, where a product is one or two rounds of warps, only for few
+// cases. us in a graph with one / two: 3,072 elements, R = 4: 6.7 / 6.7, R = 24: 10.2 / 11.2;
+// 7,986, R = 6: 9.6 / 9.1, R = 16: 13.5 / 15.5; 16,464, R = 8: 14.3 / 15.4, R = 32: 39.3 / 40.3;
+// 31,104, R = 6: 22.4 / 20.9, R = 32: 67.8 / 67.0; 146,124, R = 32: 336 / 315.
+inline bool direct_two_cases(int64_t n_elem, int R) { return R % 2 == 0 && (R <= 6 || n_elem >= 24000); }
+
 // Rounds that `warps` warps of equal length take on the 4 * sms SM sub-partitions, each of
 // which runs its warps through its FP64 unit one instruction after the other: the number on
 // the fullest one. (Fewer warps than sub-partitions do not go one to each: some share one.)

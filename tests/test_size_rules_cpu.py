@@ -16,6 +16,7 @@ SMS = 152
 HARNESS = r"""
 #include "fe_rules.cuh"
 extern "C" int four_case_passes(long n, int R, int sms) { return fe::four_case_passes(n, R, sms); }
+extern "C" int direct_two_cases(long n, int R) { return fe::direct_two_cases(n, R); }
 extern "C" int f64_direct_split(long n, int R, int sms) { return fe::f64_direct_split(n, R, sms); }
 extern "C" int f64_adjoint_split(long n, int R, int sms) { return fe::f64_adjoint_split(n, R, sms); }
 """
@@ -51,6 +52,23 @@ def test_passes_of_four_cases(rules, n, R, one, four):
 @pytest.mark.parametrize("R", [1, 2, 6, 13])
 def test_passes_of_four_cases_need_a_multiple_of_four(rules, R):
     assert not rules.four_case_passes(ctypes.c_long(10**7), R, SMS)
+
+
+# us per FP32 direct product with one case and with two cases per thread (to 4 %: between the
+# smallest and largest meshes the two are as near to each other as that)
+@pytest.mark.parametrize("n_elem,R,one,two", [
+    (750, 16, 6.5, 6.4), (3072, 4, 6.7, 6.7), (3072, 24, 10.2, 11.2), (3072, 48, 14.7, 16.0), (7986, 6, 9.6, 9.1),
+    (7986, 16, 13.5, 15.5), (7986, 64, 38.6, 40.3), (16464, 2, 10.3, 9.3), (16464, 8, 14.3, 15.4),
+    (16464, 18, 28.2, 27.7), (16464, 32, 39.3, 40.3), (31104, 6, 22.4, 20.9), (31104, 16, 38.7, 39.9),
+    (31104, 28, 67.5, 64.5), (73728, 2, 22.8, 20.3), (73728, 32, 166.4, 158.4), (146124, 32, 336.1, 315.3)])
+def test_cases_per_thread_of_the_fp32_product(rules, n_elem, R, one, two):
+    times = {0: one, 1: two}
+    assert times[rules.direct_two_cases(ctypes.c_long(n_elem), R)] <= 1.04 * min(one, two)
+
+
+@pytest.mark.parametrize("R", [1, 3, 7, 31])
+def test_two_cases_need_an_even_number(rules, R):
+    assert not rules.direct_two_cases(ctypes.c_long(10**6), R)
 
 
 # us per FP64 direct product by lanes per element (0: a lane per corner), the fastest few
