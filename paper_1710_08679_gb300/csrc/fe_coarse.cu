@@ -427,9 +427,12 @@ __device__ __forceinline__ void add_term(const SlicedTerm& t, float acc[12]) {
 // one sector for 8 rows (from the plain [nnzb][9] layout each read 8 sectors: ncu
 // showed the L1 88 % busy and 13 sectors per load request). The column and x are a
 // dependent pair of loads and the kernel waits on little else, so two blocks are in
-// flight at a time; 64 registers keep eight 128-thread CTAs on an SM (R = 16 on the 70x70x35
-// crust block: 57.4 -> 56.1 us).
-__global__ void __launch_bounds__(128, 8) spmv4_sliced_kernel(int64_t N4, int R, const int32_t* __restrict__ rowptr,
+// flight at a time (PAIRS; level1_two_blocks) where 64 registers a thread leave room
+// for enough threads; the values are loaded while the columns are on their way. R = 16 on the
+// 70x70x35 crust block in a graph: 55.4 us with one block in flight, 52.8 us with two.
+template <bool PAIRS>
+__global__ void __launch_bounds__(64, PAIRS ? 16 : 20) spmv4_sliced_kernel(int64_t N4, int R,
+                                                                const int32_t* __restrict__ rowptr,
                                                                 const int32_t* __restrict__ sl_off,
                                                                 const int32_t* __restrict__ sl_cols,
                                                                 const float* __restrict__ sl_vals,
@@ -450,20 +453,21 @@ __global__ void __launch_bounds__(128, 8) spmv4_sliced_kernel(int64_t N4, int R,
   const int32_t* c = sl_cols + base * 8 + rr;
   const float* B = sl_vals + base * 72 + rr;
   int t = 0;
-  for (; t + 1 < len; t += 2, c += 16, B += 144) {
+  for (; PAIRS && t + 1 < len; t += 2, c += 16, B += 144) {
     const int64_t b0 = __ldg(c), b1 = __ldg(c + 8);
     SlicedTerm t0, t1;
-    load_x(t0, x, b0, R, r0);
-    load_x(t1, x, b1, R, r0);
     load_m(t0, B);
     load_m(t1, B + 72);
+    load_x(t0, x, b0, R, r0);
+    load_x(t1, x, b1, R, r0);
     add_term(t0, acc);
     add_term(t1, acc);
   }
-  if (t < len) {
+  for (; t < len; ++t, c += 8, B += 72) {
     SlicedTerm t0;
-    load_x(t0, x, __ldg(c), R, r0);
+    const int64_t b = __ldg(c);
     load_m(t0, B);
+    load_x(t0, x, b, R, r0);
     add_term(t0, acc);
   }
   float4* o = reinterpret_cast<float4*>(y + (a * R + r0) * 3);
@@ -785,7 +789,10 @@ void coarse_spmv(const fe_mesh* m, int R, const float* x4, float* y4, cudaStream
   const Coarse& c = m->coarse;
   FE_REQUIRE(c.csr_ready, "coarse matrix not assembled");
   if (R % 4 == 0 && c.sl_vals.ptr) {
-    spmv4_sliced_kernel<<<(unsigned)((c.n_nodes * (R / 4) + 127) / 128), 128, 0, s>>>(
+    int sms = 0;
+    FE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
+    auto kern = level1_two_blocks(c.n_nodes, R, sms) ? spmv4_sliced_kernel<true> : spmv4_sliced_kernel<false>;
+    kern<<<(unsigned)((c.n_nodes * (R / 4) + 63) / 64), 64, 0, s>>>(
         c.n_nodes, R, c.rowptr.as<int32_t>(), c.sl_off.as<int32_t>(), c.sl_cols.as<int32_t>(), c.sl_vals.as<float>(),
         x4, y4, skip);
     FE_CHECK_LAUNCH();

@@ -65,6 +65,17 @@ inline int f64_adjoint_split(int64_t n_elem, int R, int sms) {
   return f64_case_split(n_elem, R, 500, 110, sms, true);
 }
 
+// Level-1 product from the sliced matrix: two blocks of a row in flight (64 registers, 1,024
+// threads per SM) or one (48 registers, 1,280). Two cover more latency, one fits a few more
+// threads: it is the faster one where it takes a round of threads less. us in a graph with
+// one / two by w, the rounds of threads with two: w = 0.56 8.3 / 7.7; w = 1.17 25.0 / 28.6;
+// w = 1.26 13.7 / 14.8; w = 1.36 16.4 / 16.2; w = 2.33 34.9 / 35.9; w = 2.44 21.8 / 23.3;
+// w = 2.71 25.7 / 25.2; w = 4.66 56.1 / 52.8; w = 9.33 98.1 / 90.5.
+inline bool level1_two_blocks(int64_t n_nodes, int R, int sms) {
+  const double w = (double)(n_nodes * (R / 4)) / (1024.0 * sms);
+  return !((w > 1.0 && w <= 1.3) || (w > 2.0 && w <= 2.5));
+}
+
 // Inner-loop vector passes with four cases per thread: from 140 such threads per SM on.
 // With fewer the SMs are filled better by a thread per case. Step of the inner loop at level
 // 0 with one / four cases per thread: 1,331 nodes, R = 4: 24.0 / 26.1 us, R = 64: 29.7 / 29.0;

@@ -17,6 +17,7 @@ HARNESS = r"""
 #include "fe_rules.cuh"
 extern "C" int four_case_passes(long n, int R, int sms) { return fe::four_case_passes(n, R, sms); }
 extern "C" int direct_two_cases(long n, int R) { return fe::direct_two_cases(n, R); }
+extern "C" int level1_two_blocks(long n, int R, int sms) { return fe::level1_two_blocks(n, R, sms); }
 extern "C" int f64_direct_split(long n, int R, int sms) { return fe::f64_direct_split(n, R, sms); }
 extern "C" int f64_adjoint_split(long n, int R, int sms) { return fe::f64_adjoint_split(n, R, sms); }
 """
@@ -69,6 +70,17 @@ def test_cases_per_thread_of_the_fp32_product(rules, n_elem, R, one, two):
 @pytest.mark.parametrize("R", [1, 3, 7, 31])
 def test_two_cases_need_an_even_number(rules, R):
     assert not rules.direct_two_cases(ctypes.c_long(10**6), R)
+
+
+# us per level-1 product with one and with two blocks of a row in flight
+@pytest.mark.parametrize("n,R,one,two", [
+    (6825, 64, 8.4, 8.3), (10875, 64, 10.8, 12.6), (14025, 48, 11.2, 12.8), (14025, 56, 13.7, 14.8),
+    (14025, 64, 15.0, 14.4), (21793, 64, 19.1, 20.1), (27132, 28, 12.8, 14.8), (27132, 56, 21.8, 23.3),
+    (42189, 16, 11.5, 13.3), (42189, 20, 16.4, 16.2), (59625, 32, 30.1, 27.3), (83997, 8, 12.6, 14.1),
+    (83997, 20, 32.5, 29.8), (181476, 4, 25.0, 28.6), (181476, 8, 34.9, 35.9), (181476, 12, 46.6, 45.3),
+    (181476, 16, 56.1, 52.8), (181476, 64, 176.2, 167.7)])
+def test_blocks_in_flight_of_the_level1_product(rules, n, R, one, two):
+    assert near_best(rules.level1_two_blocks(ctypes.c_long(n), R, SMS), {0: one, 1: two})
 
 
 # us per FP64 direct product by lanes per element (0: a lane per corner), the fastest few
