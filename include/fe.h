@@ -76,9 +76,14 @@ typedef struct {
   int32_t max_outer;     /* cap on outer iterations (PCG64: CG iterations) */
   int32_t n_inner;       /* cap on inner steps per outer iteration (30) */
   double eps_inner;      /* inner stop: max over active cases ||e||^2/||rbar||^2 <= eps_inner (0.1) */
-  int32_t use_graph;     /* 1: replay one outer iteration from a captured CUDA graph */
+  int32_t use_graph;     /* 1: replay one outer iteration from a captured CUDA graph (PCG64 with
+                            check_every 1: iterations until a case leaves, see there) */
   int32_t literal_beta;  /* 1: the printed beta = (z,q)/rho; 0: flexible CG beta (default) */
-  int32_t check_every;   /* outer iterations between host reads of the convergence flags (>= 1) */
+  int32_t check_every;   /* outer iterations between host reads of the convergence flags (>= 1).
+                            PCG64 with use_graph and 1 (the default): the graph repeats the
+                            iteration on the device until a case converges, breaks down or
+                            reaches max_outer, and the host reads the flags then; the same
+                            iterates. Larger values replay and read single iterations */
   int32_t verbose;       /* reserved, 0 */
   int32_t n_inner1;      /* FCG_MG: cap on level-1 (TET4) inner steps per outer iteration (300) */
   double eps_inner1;     /* FCG_MG: level-1 inner stop, the same rule as eps_inner (0.05) */
