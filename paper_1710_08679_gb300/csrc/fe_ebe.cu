@@ -240,11 +240,10 @@ __global__ void __launch_bounds__(32) ebe_direct_f64_kernel(MeshView<double> M, 
 // FP64 direct kernel for few items: four lanes per (element, case), lane m = corner m. A
 // warp's FP64 instruction occupies its SM sub-partition for some 60 cycles whatever the
 // other sub-partitions do, so with fewer warps than sub-partitions (608) the time is one
-// warp's FP64 instruction count: about 550 with a lane per element. Here a lane forms its
+// warp's FP64 instruction count: about 530 with a lane per element (ncu). Here a lane forms its
 // corner's gradient, stress s_m, corner output and its terms T_m g_l of the three edges at
-// its corner: about 185. One case on the 3,072 elements of the 8^3 box: 25 us with a lane per
-// element (kernel); the whole product 28.3 (gather kernel, the fastest before) -> 18.1 us; a
-// 172-step PCG solve 7.6 -> 5.1 ms.
+// its corner: 170. One case on the 3,072 elements of the 8^3 box in a graph: 23.1 us with a lane
+// per element, 11.5 us here; a 172-step PCG solve 7.6 and 5.1 ms.
 __global__ void __launch_bounds__(64) ebe_corner_f64_kernel(MeshView<double> M, int R,
                                                             const uint16_t* __restrict__ own,
                                                             const double* __restrict__ x, double* __restrict__ y,
@@ -1810,7 +1809,7 @@ template void ebe_apply<float>(const fe_mesh*, int, const float*, float*, cudaSt
 template void ebe_apply<double>(const fe_mesh*, int, const double*, double*, cudaStream_t, const int*);
 
 // Times each candidate kernel for (R, precision) on this mesh (scratch vectors
-// of ones, 2 warm-up and 5 timed products each, CUDA events on `s`) and keeps
+// of zeros, 2 warm-up and 5 timed products each, CUDA events on `s`) and keeps
 // the fastest. Candidates, where the tile's shared-memory footprint fits: direct;
 // gather with 12..256 elements per tile; tiled with 24..96; for FP64 the
 // float-float gather with 4..24; for FP32 the paired-arithmetic gather with 16..96

@@ -814,9 +814,9 @@ void ws_wait_selftest(const fe_mesh* m, long long cycles, cudaStream_t s) {
   FE_CHECK_LAUNCH();
 }
 
-// Every multiple of 4 up to 32 (node rows are 16-byte vectors of four cases). Before, R =
-// 12, 20, 24 and 28 had only the direct and tiled kernels: on the 41x33x18 crust block
-// 146 / 256 / 287 / 347 us per product, now 95 / 145 / 163 / 199 us.
+// Every multiple of 4 up to 32: node rows are 16-byte vectors of four cases. R = 12 / 20 / 24 /
+// 28 on the 41x33x18 crust block: 146 / 256 / 287 / 347 us with the fastest other kernel, 95 /
+// 145 / 163 / 199 us with this one.
 bool ws_supported(int R) { return R % 4 == 0 && R >= 4 && R <= 32; }
 
 // Loader warps of a block with sw staging warps (one geometry warp, the rest sum nodes).

@@ -701,10 +701,9 @@ __global__ void k_outer_update(int64_t N, Cases C, double* __restrict__ rv, cons
 // The FP64 passes of an outer iteration for even R: thread = (node, 2 cases), 48 contiguous
 // bytes of an FP64 vector in three 16-byte loads. Same arithmetic per value as k_outer_zq,
 // k_dot, k_outer_update and k_cast_start. Bound by HBM once the FP64 pipe has only the
-// multiply-adds to do. R = 16, 1.41 M nodes: (z, q) 0.30, (z, r) and (p, q) 0.38, update 0.66,
-// start 0.25 ms before; (z, q) and (z, r) 0.25, (p, q) 0.15, update 0.53, start 0.18 ms now.
-// (k_outer_p
-// in this form took 0.34 instead of 0.24 ms and stays with one case per thread.)
+// multiply-adds to do. R = 16, 1.41 M nodes: update 0.66 ms with one case per thread, 0.53 ms
+// here, start 0.25 and 0.18 ms; (z, q) and (z, r) together 0.25, (p, q) 0.15 ms. (k_outer_p in
+// this form takes 0.34 instead of 0.24 ms and stays with one case per thread.)
 __global__ void __launch_bounds__(256) k_outer_zq2(int64_t N, Cases C, const float* __restrict__ ub,
                                                    const double* __restrict__ q, const double* __restrict__ rv) {
   extern __shared__ double sm[];
